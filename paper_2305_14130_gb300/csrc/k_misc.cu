@@ -6,7 +6,7 @@
 #include <cmath>
 
 #include "plan.hpp"
-#include "reg_pixel.cuh"
+#include "reg_block.cuh"
 
 namespace efwi {
 namespace {
@@ -378,37 +378,24 @@ __global__ void k_zoi(ZoiShot z, int s, int nx, int nz, double dx, double dz, do
     sink[o] = inside ? 1 : 0;
 }
 
-// Consistency term per pixel: reg_pixel (reg_pixel.cuh).
-// Collapse of an extended field to one physical field (eq. 9, and eq. 15 when
-// applied to the per-source gradients): out = S_w W x~ per pixel, FP64:
-//   (W x)_s = (d_s - c_s b_s) x_s + c_s sum_i b_i x_i  (eq. 11, c_s and d_s as in k_reg)
-//   out = sum_s b'_s (W x)_s / sum_s b'_s               (eq. 12)
-__global__ void k_collapse(const float *x, const float *b, const float *bp, const uint8_t *sink, int ns,
-                           long long npix, float *out) {
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += (long long)gridDim.x * blockDim.x) {
-        double B = 0, BX = 0, SBp = 0;
-        for (int s = 0; s < ns; ++s) {
-            const long long o = s * npix + p;
-            B += b[o]; BX += (double)b[o] * x[o]; SBp += bp[o];
-        }
-        double acc = 0;
-        for (int s = 0; s < ns; ++s) {
-            const long long o = s * npix + p;
-            const double bs = b[o];
-            const bool in = sink[o] != 0 && ns > 1;
-            const double c = in ? (1.0 - bs) / (B - bs) : 0.0;
-            const double dd = in ? bs : 1.0;
-            acc += (double)bp[o] * ((dd - c * bs) * x[o] + c * BX);
-        }
-        out[p] = (float)(acc / SBp);
-    }
+// Consistency term and collapse (eq. 9; eq. 15 when applied to the per-source gradients): 32
+// pixels per block and iteration (reg_block.cuh).
+template <int CPT>
+__global__ void __launch_bounds__(kRegThreads, reg_blocks(CPT)) k_collapse(const float *x, const float *b, const float *bp,
+                                                          const uint8_t *sink, int ns, long long npix, float *out) {
+    __shared__ RegShared sh;
+    for (long long p0 = (long long)blockIdx.x * kRegPx; p0 < npix; p0 += (long long)gridDim.x * kRegPx)
+        reg_block<CPT, true>(x, b, bp, sink, ns, npix, p0, 0.0, nullptr, out, sh);
 }
 
-__global__ void k_reg(const float *m, const float *b, const float *bp, const uint8_t *sink, int ns, long long npix,
-                      double eta2, float *g, double *partial) {
+template <int CPT>
+__global__ void __launch_bounds__(kRegThreads, reg_blocks(CPT)) k_reg(const float *m, const float *b, const float *bp,
+                                                     const uint8_t *sink, int ns, long long npix, double eta2,
+                                                     float *g, double *partial) {
+    __shared__ RegShared sh;
     double acc = 0.0;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += (long long)gridDim.x * blockDim.x)
-        acc += reg_pixel(m, b, bp, sink, ns, npix, p, eta2, g);
+    for (long long p0 = (long long)blockIdx.x * kRegPx; p0 < npix; p0 += (long long)gridDim.x * kRegPx)
+        acc += reg_block<CPT, false>(m, b, bp, sink, ns, npix, p0, eta2, g, nullptr, sh);
     acc = block_sum(acc);
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
@@ -579,17 +566,35 @@ int launch_zoi(int ns, int nx, int nz, double dx, double dz, const efwi_zoi_desc
     return EFWI_OK;
 }
 
+// blocks of a grid-stride pass over npix pixels: all resident at once, at most `most`
+static int reg_grid(const void *kernel, long long npix, int most) {
+    int dev = 0, sms = 1, nb = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kRegThreads, 0);
+    return (int)std::max<long long>(1, std::min<long long>((npix + kRegPx - 1) / kRegPx,
+                                                           std::min(std::max(nb, 1) * sms, most)));
+}
+
 void launch_collapse(int ns, long long npix, const float *x, const float *b, const float *bp, const uint8_t *sink,
                      float *out, cudaStream_t st) {
-    const long long blocks = std::min<long long>((npix + 255) / 256, 152LL * 16);
-    k_collapse<<<(int)std::max<long long>(blocks, 1), 256, 0, st>>>(x, b, bp, sink, ns, npix, out);
+    reg_dispatch(ns, [&](auto cpt) {
+        constexpr int C = decltype(cpt)::value;
+        const int grid = reg_grid((const void *)k_collapse<C>, npix, 1 << 16);
+        k_collapse<C><<<grid, kRegThreads, 0, st>>>(x, b, bp, sink, ns, npix, out);
+    });
 }
 
 void launch_reg(efwi_plan *p, const float *m, const float *b, const float *bp, const uint8_t *sink, double eta,
                 double *phi, float *g, int accumulate_phi, cudaStream_t st, int ns) {
     const long long npix = (long long)p->d.nz * p->d.nx;
-    k_reg<<<kPartials, kRedThreads, 0, st>>>(m, b, bp, sink, ns > 0 ? ns : p->d.ns, npix, eta * eta, g, p->partial);
-    k_final_sum<<<1, 1024, 0, st>>>(p->partial, kPartials, 0.5 * eta * eta, phi, accumulate_phi);
+    if (ns <= 0) ns = p->d.ns;
+    reg_dispatch(ns, [&](auto cpt) {
+        constexpr int C = decltype(cpt)::value;
+        const int grid = reg_grid((const void *)k_reg<C>, npix, kPartials);
+        k_reg<C><<<grid, kRegThreads, 0, st>>>(m, b, bp, sink, ns, npix, eta * eta, g, p->partial);
+        k_final_sum<<<1, 1024, 0, st>>>(p->partial, grid, 0.5 * eta * eta, phi, accumulate_phi);
+    });
     p->launches += 2;
 }
 

@@ -20,18 +20,19 @@
 // share the array: calls that overlap on the GPU (different streams, or host
 // threads racing on one device) race on it.  Every call writes all the
 // partials it later reads, so nothing has to be cleared between calls.
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <string>
 
 #include "plan.hpp"
-#include "reg_pixel.cuh"
+#include "reg_block.cuh"
 
 namespace {
 
-constexpr int kNaThreads = 256;
+constexpr int kNaThreads = efwi::kRegThreads;
 constexpr int kNaBlocks = 4096;                                   // partials held by the scratch array
-constexpr long long kNaMaxPixels = (long long)kNaBlocks * kNaThreads;   // one pixel per thread
+constexpr long long kNaMaxPixels = (long long)kNaBlocks * 256;    // the entry point's documented limit
 
 static __device__ __align__(256) double g_na_partials[kNaBlocks];
 
@@ -50,13 +51,15 @@ __device__ double na_block_sum(double v) {
     return v;
 }
 
-// One pixel per thread; the per-pixel arithmetic of eqs. 8, 11, 12 is
-// reg_pixel, the same as the plan's kernel.
-__global__ void k_reg_noalloc(const float *m, const float *b, const float *bp, const uint8_t *sink, int ns,
-                              long long npix, double eta2, float *g, double *partial) {
-    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// The arithmetic of eqs. 8, 11, 12 is reg_block, the same as the plan's kernel.
+template <int CPT>
+__global__ void __launch_bounds__(kNaThreads, efwi::reg_blocks(CPT)) k_reg_noalloc(const float *m, const float *b, const float *bp,
+                                                            const uint8_t *sink, int ns, long long npix, double eta2,
+                                                            float *g, double *partial) {
+    __shared__ efwi::RegShared sh;
     double acc = 0.0;
-    if (p < npix) acc = efwi::reg_pixel(m, b, bp, sink, ns, npix, p, eta2, g);
+    for (long long p0 = (long long)blockIdx.x * efwi::kRegPx; p0 < npix; p0 += (long long)gridDim.x * efwi::kRegPx)
+        acc += efwi::reg_block<CPT, false>(m, b, bp, sink, ns, npix, p0, eta2, g, nullptr, sh);
     acc = na_block_sum(acc);
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
@@ -136,8 +139,11 @@ extern "C" int efwi_regularization_grad_noalloc(int ns, int nx, int nz, const fl
         efwi::set_thread_error(err);
         return rc;
     }
-    const int blocks = (int)((npix + kNaThreads - 1) / kNaThreads);
-    k_reg_noalloc<<<blocks, kNaThreads, 0, st>>>(m, b, bp, sink, ns, npix, eta * eta, g, partial);
+    const int blocks = (int)std::min<long long>((npix + efwi::kRegPx - 1) / efwi::kRegPx, kNaBlocks);
+    efwi::reg_dispatch(ns, [&](auto cpt) {
+        k_reg_noalloc<decltype(cpt)::value><<<blocks, kNaThreads, 0, st>>>(m, b, bp, sink, ns, npix, eta * eta, g,
+                                                                          partial);
+    });
     k_sum_noalloc<<<1, 1024, 0, st>>>(partial, blocks, 0.5 * eta * eta, phi_reg);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
