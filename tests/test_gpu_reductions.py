@@ -1,5 +1,6 @@
 """Reductions formed in FP32 with their rounding errors carried along: the consistency term and
-the collapse over every branch of their component split, against FP64."""
+the collapse over every branch of their component split, and the l-BFGS inner products over
+tails, alignments and magnitudes, against FP64."""
 import numpy as np
 import pytest
 import torch
@@ -7,6 +8,7 @@ import torch
 import workloads as W
 from common import f32, rel_l2
 from oracle import extension as X
+from oracle import lbfgs as L
 
 pytestmark = pytest.mark.gpu
 
@@ -67,3 +69,28 @@ def test_consistency_term_keeps_non_finite_values_to_their_pixel(efwi):
     assert np.isnan(phi.item())
     assert bad[:, 2, 40].all() and bad[:, 1, 7].all() and bad.sum() == 2 * ns
     plan.close()
+
+
+# tails of a block's 2048 elements, one element, more than one pass of the 1216-block grid; the
+# caller's gradient and direction 16-byte aligned or not; magnitudes whose products leave FP32
+@pytest.mark.parametrize("scale", [1.0, 1e-24, 1e16])
+@pytest.mark.parametrize("n,shift", [(1, 0), (7, 1), (2047, 0), (2049, 3), (2_490_373, 1)])
+def test_direction_over_tails_alignments_and_magnitudes(efwi, n, shift, scale):
+    from paper_2305_14130_gb300.optim import LBFGS
+    rng = np.random.default_rng(n)
+    a = rng.uniform(0.5, 5.0, n)
+    S = np.float32(scale * rng.standard_normal((3, n)))
+    Y = np.float32(S * a)
+    g = np.float32(scale * rng.standard_normal(n))
+    opt = LBFGS(n, m=3)
+    for s, y in zip(S, Y):
+        assert opt.push(dev(s), dev(y))
+    gd = torch.zeros(n + 4, device="cuda")[shift:shift + n]
+    gd.copy_(dev(g))
+    d = opt.direction(gd).cpu().numpy()
+    ref = -L.two_loop(g.astype(np.float64), S.astype(np.float64), Y.astype(np.float64))
+    assert rel_l2(d, ref) <= 1e-5
+    # in place: the caller's gradient becomes the direction
+    opt.direction(gd, gd)
+    assert np.array_equal(gd.cpu().numpy(), d)
+    opt.close()
