@@ -273,10 +273,12 @@ typedef struct efwi_zoi_desc {
  * are bitwise the same for every variant of one adjoint form):
  *   EFWI_TMA_STAGES=n     the autotuner keeps only n-stage TMA forward variants
  *   EFWI_TMA_VEC=v        only forward layout v (1 single cells, 2 cell pairs,
- *                         3 cell pairs with the halo ring as single cells)
+ *                         3 cell pairs with the halo ring as single cells,
+ *                         4, 5 packed cell pairs, tiles from a counter / at a stride)
  *   EFWI_ADJ_PERSIST=0|1  only the one-CTA-per-tile / persistent-grid adjoint
- *   EFWI_ADJ_VEC=1|2|3    only the single-cell / cell-pair / 512-thread cell-pair TMA
- *                         scaled-stress adjoint
+ *   EFWI_ADJ_VEC=1|..|5    only the single-cell / cell-pair / 512-thread cell-pair /
+ *                         packed cell-pair (4, 5 as above) TMA scaled-stress
+ *                         adjoint
  *   EFWI_PREFETCH=0|1     L2 prefetch one tile ahead off / on (else timed)
  *   EFWI_AUTOTUNE_LOG=1   print every timed variant on stderr
  *   EFWI_TEST_FAIL_ALLOC=k  make the k-th workspace allocation fail with

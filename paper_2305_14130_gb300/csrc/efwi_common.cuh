@@ -35,7 +35,7 @@
 #define EFWI_FLAG_SELFTEST 4     // the timeout self-test's wait expired (as intended)
 #define EFWI_FLAG_SHEAR 8        // a gradient call met mu <= 0 (or lambda + mu <= 0, scaled-stress adjoint)
 
-#define EFWI_GX 4
+#define EFWI_GX 8
 #define EFWI_GZ 2
 
 namespace efwi {

@@ -767,7 +767,7 @@ int efwi_autotune(efwi_plan *p) {
     for (auto &s : kShapes) {
         if (fixed && (s.tx != p->tile_x || s.tz != p->tile_z)) continue;
         if (want == EFWI_STENCIL_AUTO || want == EFWI_STENCIL_LOADS) fwd.push_back({EFWI_STENCIL_LOADS, s.tx, s.tz, 0});
-        for (int vec = 1; vec <= 3; ++vec)
+        for (int vec = 1; vec <= (tile_ok(p) ? 5 : 3); ++vec)
             for (int stg = 0; stg <= 1; ++stg) {
                 const int kind = vec == 1 ? EFWI_STENCIL_TMA : stg ? EFWI_STENCIL_TMA_STAGED : EFWI_STENCIL_TMA_PAIRS;
                 if (want != EFWI_STENCIL_AUTO && want != kind) continue;
@@ -803,7 +803,7 @@ int efwi_autotune(efwi_plan *p) {
         const char *fa = getenv("EFWI_ADJ_VEC");
         const int only_av = fa ? atoi(fa) : 0;
         if (want_a != EFWI_STENCIL_LOADS && adj_scaled_tma_shape_ok(s.tx, s.tz))
-            for (int av = 1; av <= 3; ++av)   // 3: cell pairs, 512-thread CTAs
+            for (int av = 1; av <= (tile_ok(p) ? 5 : 3); ++av)   // 3: 512-thread CTAs; 4, 5: packed pairs
                 if (!only_av || av == only_av) adj.push_back({EFWI_STENCIL_TMA, s.tx, s.tz, 2, av});
     }
     if (scaled && adj.empty()) {
@@ -882,7 +882,7 @@ int efwi_autotune(efwi_plan *p) {
         const char *fe = getenv("EFWI_PREFETCH");
         const int force_pf = fe ? atoi(fe) : -1;
         p->tma_pf = p->adj_pf = 0;
-        const bool fwd_ok = !rc && p->stencil >= EFWI_STENCIL_TMA;
+        const bool fwd_ok = !rc && p->stencil >= EFWI_STENCIL_TMA && p->tma_vec < 4;
         const bool adj_ok = !rc && p->adj_stencil == EFWI_STENCIL_LOADS && p->adj_grid > 0 &&
                             p->adj_form == EFWI_ADJ_FORM_STRESS &&
                             tma_encode_adj_maps(p, p->adj_tile_x, p->adj_tile_z) == EFWI_OK;

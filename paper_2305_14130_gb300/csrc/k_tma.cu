@@ -22,71 +22,12 @@
 
 #include "plan.hpp"
 #include "tma.cuh"
+#include "fwd_tile.cuh"
 
 namespace efwi {
 namespace {
 
 constexpr int kThreads = 256;
-
-struct TmaFwdArgs {
-    const ShotDev *shots;
-    const int4 *tiles;
-    const FwdMaps *maps;
-    int ntiles;
-    int scur;                   // state buffer read (z offset 5 * scur in the state map)
-    Fields out;                 // state buffer written
-    Pml pml;                    // V block = current (read), S block = in place
-    float *n1, *n3, *n2, *n4;   // next V block
-    float *segx, *segz;
-    const float *dw;
-    const float *wv;            // w_n / (dx dz) of force sources (null without)
-    int nt, n;
-    float dt, rdx, rdz;
-    int *err;
-    int ofield;                 // state-map field of the written buffer's vx (output staging)
-    int segf;                   // segment-map field of this step's vx, or -1 (output staging)
-    SnapW sw;                   // reduced-precision snapshot work (sw.h / sw.amax null: none)
-    int pf;                     // 1: L2 prefetch of the tile one beyond the shared-memory pipeline
-};
-
-// Shared-memory stage of one tile.  Fields are staged on the tile + 4-cell halo in x
-// (SX columns) and, in z, only on the rows their readers use (halo-4 row coordinates,
-// rows 0 .. TZ+7): vx, vz, sigma_xx, b_x, b_z on rows 2 .. TZ+5 (R2 rows), sigma_zz on
-// rows 1 .. TZ+7 and sigma_xz on rows 0 .. TZ+6 (R3 rows each); lambda, mu, mu_xz on the
-// tile.  Every array starts 128-byte aligned; vx|vz and b_x|b_z are 2-field boxes.
-template <int TX, int TZ, int NST, int VEC = 1>
-struct FwdLayout {
-    static constexpr int SX = TX + 8, SZ = TZ + 8;
-    static constexpr int R2 = TZ + 4, R3 = TZ + 7;
-    static constexpr int A2 = SX * R2;                              // floats of an R2 field
-    static constexpr int A3 = SX * R3, A3P = (A3 + 31) & ~31;       // R3 field, padded to 128 B
-    static constexpr int NC = TX * TZ;                              // one tile field
-    static constexpr int OVX = 0, OVZ = A2, OSXX = 2 * A2, OSZZ = 3 * A2, OSXZ = OSZZ + A3P,
-                         OBX = OSXZ + A3P, OBZ = OBX + A2, OLAM = OBZ + A2;
-    static constexpr int BUF = (OLAM + 3 * NC + 31) & ~31;          // floats per stage
-    static constexpr unsigned LOADED = (5u * A2 + 2u * A3 + 3u * NC) * 4u;   // bytes the copies bring
-    static constexpr size_t smem() { return NST * (size_t)BUF * 4 + 128; }
-    static_assert(A2 % 32 == 0, "R2 fields must keep 128-byte alignment");
-    static_assert(2 * NC <= 2 * A2, "staged velocities must fit over b_x, b_z");
-};
-
-// tl: the tile's work item, already in a register (the issuing thread's refill then has no
-// dependent global load between the tile's barriers)
-template <int TX, int TZ, int NST, int VEC>
-__device__ __forceinline__ void issue_fwd(const TmaFwdArgs &a, const int4 tl, float *buf, uint64_t *bar) {
-    using L = FwdLayout<TX, TZ, NST, VEC>;
-    const FwdMaps *m = a.maps + tl.x;
-    mbar_expect_tx(bar, L::LOADED);
-    // element x = cell i + GX (halo-4 column 0 = cell i0 - 4), row y = cell j + GZ: halo-4 row r
-    // of the tile is map row j0 - 4 + r + GZ = tl.z - 2 + r
-    const int f = 5 * a.scur;
-    tma_load_3d(buf + L::OVX, &m->s2, bar, tl.y, tl.z, f);          // vx, vz: rows 2..
-    tma_load_3d(buf + L::OSXX, &m->s1, bar, tl.y, tl.z, f + 2);     // sigma_xx: rows 2..
-    tma_load_3d(buf + L::OSZZ, &m->s3, bar, tl.y, tl.z - 1, f + 3); // sigma_zz: rows 1..
-    tma_load_3d(buf + L::OSXZ, &m->s3, bar, tl.y, tl.z - 2, f + 4); // sigma_xz: rows 0..
-    tma_load_3d(buf + L::OBX, &m->mb, bar, tl.y, tl.z, 3);          // b_x, b_z: rows 2..
-    tma_load_3d(buf + L::OLAM, &m->mc, bar, tl.y + 4, tl.z + 2, 0); // lambda, mu, mu_xz: tile
-}
 
 // The boxes issue_fwd copies, brought into L2 only (a tile beyond the pipeline).
 __device__ __forceinline__ void prefetch_fwd(const TmaFwdArgs &a, int4 tl) {
@@ -680,6 +621,7 @@ int encode_map(CUtensorMap *m, void *base, const ShotDev &s, long long F, int nf
 }
 
 bool tma_shape_ok(int tx, int tz, int nst, int vec, int st, int snap) {
+    if (vec >= 4) return vec <= 5 && tx == 32 && tz == 16 && nst == 2 && st == 0;
 #define EFWI_OK_X(a, b, c, d, e) if (tx == a && tz == b && nst == c && vec == d && st == e) return true;
     if (snap != EFWI_STORE_FP32) {
         EFWI_TMA_SNAP_VARIANTS(EFWI_OK_X)
@@ -720,7 +662,8 @@ int tma_prepare_fwd(efwi_plan *p, int tx, int tz, int nst, int vec, int stg) {
     if (tx == a && tz == b && nst == c && vec == d && stg == e)                                        \
         nb = sk == EFWI_STORE_FP16 ? occupancy<a, b, c, d, e, EFWI_STORE_FP16>()                       \
                                    : occupancy<a, b, c, d, e, EFWI_STORE_BF16>();
-    if (sk == EFWI_STORE_FP32) { EFWI_TMA_VARIANTS(EFWI_OCC_X) }
+    if (vec >= 4) nb = tile_blocks_per_sm(sk, vec);
+    else if (sk == EFWI_STORE_FP32) { EFWI_TMA_VARIANTS(EFWI_OCC_X) }
     else { EFWI_TMA_SNAP_VARIANTS(EFWI_OCC_SNAP_X) }
 #undef EFWI_OCC_X
 #undef EFWI_OCC_SNAP_X
@@ -734,7 +677,7 @@ int tma_prepare_fwd(efwi_plan *p, int tx, int tz, int nst, int vec, int stg) {
     return EFWI_OK;
 }
 
-void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st) {
+TmaFwdArgs tma_fwd_args(efwi_plan *p, int n, const SnapOut &so) {
     float *segx = so.fx, *segz = so.fz;
     TmaFwdArgs a;
     a.shots = p->shots_d;
@@ -755,10 +698,20 @@ void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st) {
     a.rdx = (float)(1.0 / p->d.dx);
     a.rdz = (float)(1.0 / p->d.dz);
     a.err = p->dev_err;
+    a.count = p->tile_count;
     a.ofield = 5 * (1 - p->scur);
     a.segf = segx ? (int)((segx - p->seg) / p->fsz_total) : -1;
     a.sw = so.sw;
     a.pf = p->tma_pf;
+    return a;
+}
+
+void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st) {
+    if (p->tma_vec >= 4) {
+        launch_step_tile(p, n, so, st);
+        return;
+    }
+    const TmaFwdArgs a = tma_fwd_args(p, n, so);
     const int grid = std::min(p->grid_fwd_override > 0 ? p->grid_fwd_override : p->tma_grid, a.ntiles);
     const int tx = p->tiles.tx, tz = p->tiles.tz, nst = p->tma_stages, vec = p->tma_vec, stg = p->tma_store;
     const int sk = p->snap_store;

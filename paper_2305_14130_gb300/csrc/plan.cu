@@ -283,7 +283,7 @@ static void commit_acq(efwi_plan *p, const AcqHost &h) {
 
 static void free_plan(efwi_plan *p) {
     if (!p) return;
-    void *ptrs[] = {p->shots_d, p->state[0], p->mat, p->adj[0], p->fwd_maps, p->adj_maps, p->adjs_maps, p->dev_err, p->G, p->Gtot, p->Gcmp, p->psi, p->apsi,
+    void *ptrs[] = {p->shots_d, p->state[0], p->mat, p->adj[0], p->fwd_maps, p->adj_maps, p->adjs_maps, p->dev_err, p->tile_count, p->G, p->Gtot, p->Gcmp, p->psi, p->apsi,
                     p->prof, p->dw, p->wv, p->ref, p->tr_shot, p->tr_off, p->tr_w, p->tr_acc, p->tr_coef,
                     p->gather.tgt_shot, p->gather.tgt_field, p->gather.tgt_off, p->gather.ptr, p->gather.tr,
                     p->gather.w, p->tiles.tiles, p->adj_tiles.tiles, p->resid, p->dbuf, p->partial, p->seg, p->ck.fields, p->ck.psi,
@@ -402,7 +402,7 @@ extern "C" int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *d) {
         memset(&sh, 0, sizeof sh);
         sh.P = P; sh.x0 = x0; sh.w = w;
         sh.NX = w + 2 * P; sh.NZ = NZ;
-        sh.pitch = ((sh.NX + 7) / 8) * 8 + 8;
+        sh.pitch = (sh.NX + 12 + 31) / 32 * 32;
         sh.off = off;
         off += (((long long)(NZ + 2 * EFWI_GZ) * sh.pitch + 63) / 64) * 64;
         sh.psx = psx; psx += (long long)NZ * 2 * P;
@@ -463,6 +463,7 @@ extern "C" int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *d) {
     A(&p->mat, (size_t)(5 * F), "materials");
     A(&p->adj[0], (size_t)((batched ? 10 : 5) * F), "adjoint state");
     A(&p->dev_err, (size_t)1, "device error flag");
+    A(&p->tile_count, (size_t)2, "tile counters");
     A(&p->G, (size_t)(5 * F), "imaging accumulators");
     if (batched) {
         A(&p->Gtot, (size_t)(5 * F), "Kahan totals");

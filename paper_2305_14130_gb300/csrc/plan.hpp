@@ -138,9 +138,10 @@ struct efwi_plan {
     efwi::AdjMaps *adj_maps = nullptr;
     efwi::AdjsMaps *adjs_maps = nullptr;   // [ns] tensor maps of the TMA scaled-stress adjoint
     int adjs_vec = 1;                      // its layout: 1 = one cell per thread, 2 = cell pairs,
-                                           // 3 = cell pairs in 512-thread CTAs
+                                           // 3 = cell pairs in 512-thread CTAs, 4, 5 = packed cell pairs
     int tma_adj_grid = 0, tma_adj_stages = 1;
     int adj_grid = 0;                      // per-thread-load adjoint: persistent grid (0 = one CTA per tile)
+    int *tile_count = nullptr;             // tile counters of the lean forward and adjoint steps (zero between launches)
     int *dev_err = nullptr;                // device flag: a bounded wait expired
     bool broken = false;                   // a real bounded wait expired: the plan is not used again
     int adj_tile_x = 0, adj_tile_z = 0;    // adjoint tile
@@ -211,9 +212,15 @@ void launch_adj_vel_plain(efwi_plan *p, int shot, const float *vfx, const float 
 void launch_adj_stress_plain(efwi_plan *p, int shot, const float *vfx, const float *vfz, cudaStream_t st);
 
 // --- k_tma.cu ----------------------------------------------------------------
+// layout (vec): 1 single cells, 2 cell pairs, 3 cell pairs with the halo ring as single cells, 4 5 the
+// lean form of 3 with tiles from a counter / at a fixed stride (k_tile.cu; 32 x 16, two stages)
 bool tma_shape_ok(int tx, int tz, int nst, int vec, int st, int snap);
 int tma_prepare_fwd(efwi_plan *p, int tx, int tz, int nst, int vec, int st);
 void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st);
+// --- k_tile.cu -----------------------------------------------------------------
+bool tile_ok(const efwi_plan *p);           // the lean kernels' 32-bit offsets reach every field element
+int tile_blocks_per_sm(int snap_store, int vec);
+void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st);
 bool tma_adj_shape_ok(int tx, int tz, int nst);
 int tma_prepare_adj(efwi_plan *p, int tx, int tz, int nst);
 int tma_encode_adj_maps(efwi_plan *p, int tx, int tz);
@@ -228,9 +235,13 @@ void launch_adj_scaled(efwi_plan *p, const SnapIn &si, cudaStream_t st);
 void launch_imag_unscale(efwi_plan *p, float *G, cudaStream_t st);
 // --- k_adjs_tma.cu (the same step with TMA staging, FP32 forward velocities) ----
 bool adj_scaled_tma_shape_ok(int tx, int tz);
-// tensor maps and grid; vec 1 (single cells), 2 (cell pairs), 3 (cell pairs, 512-thread CTAs)
+// tensor maps and grid; vec 1 (single cells), 2 (cell pairs), 3 (cell pairs, 512-thread CTAs),
+// 4, 5 (packed cell pairs, tiles from a counter / at a fixed stride: k_adj_tile.cu)
 int adj_scaled_tma_prepare(efwi_plan *p, int tx, int tz, int vec);
 void launch_adj_scaled_tma(efwi_plan *p, const SnapIn &si, cudaStream_t st);
+// --- k_adj_tile.cu (layouts 4, 5: the lean form) ------------------------------------
+int adj_tile_blocks_per_sm(int snap_store, int vec);
+void launch_adj_tile(efwi_plan *p, const SnapIn &si, cudaStream_t st);
 
 // --- k_fused.cu --------------------------------------------------------------
 void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st);
