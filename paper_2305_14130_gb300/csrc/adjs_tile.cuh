@@ -61,14 +61,14 @@ __device__ __forceinline__ void issue_adjs(const TmaAdjsArgs &a, const int4 tl, 
     mbar_expect_tx(bar, L::LOADED);
     // element x = cell i + GX (halo-4 column 0 = cell i0 - 4), row y = cell j + GZ: halo-4 row r
     // of the tile is map row j0 - 4 + r + GZ = tl.z - 2 + r
-    tma_load_3d(buf + L::OVX, &m->a2, bar, tl.y, tl.z, a.af);            // v^x, v^z: rows 2..
-    tma_load_3d(buf + L::OFXX, &m->a1, bar, tl.y, tl.z, a.af + 2);       // F_xx: rows 2..
-    tma_load_3d(buf + L::OFZZ, &m->a3, bar, tl.y, tl.z - 1, a.af + 3);   // F_zz: rows 1..
-    tma_load_3d(buf + L::OFXZ, &m->a3, bar, tl.y, tl.z - 2, a.af + 4);   // F_xz: rows 0..
-    tma_load_3d(buf + L::OBX, &m->mb, bar, tl.y, tl.z, 3);               // b_x, b_z: rows 2..
-    tma_load_3d(buf + L::OWX, &m->sv, bar, tl.y, tl.z, a.vf);            // forward v_x, v_z: rows 2..
-    tma_load_3d(buf + L::OLAM, &m->mc, bar, tl.y + 4, tl.z + 2, 0);      // lambda, mu, mu_xz: tile
-    tma_load_3d(buf + L::OG, &m->gi, bar, tl.y + 4, tl.z + 2, 0);        // imaging sums: tile
+    tma_load_3d(buf + L::OVX, &m->a2, bar, tl.y - 4 + EFWI_GX, tl.z, a.af);            // v^x, v^z: rows 2..
+    tma_load_3d(buf + L::OFXX, &m->a1, bar, tl.y - 4 + EFWI_GX, tl.z, a.af + 2);       // F_xx: rows 2..
+    tma_load_3d(buf + L::OFZZ, &m->a3, bar, tl.y - 4 + EFWI_GX, tl.z - 1, a.af + 3);   // F_zz: rows 1..
+    tma_load_3d(buf + L::OFXZ, &m->a3, bar, tl.y - 4 + EFWI_GX, tl.z - 2, a.af + 4);   // F_xz: rows 0..
+    tma_load_3d(buf + L::OBX, &m->mb, bar, tl.y - 4 + EFWI_GX, tl.z, 3);               // b_x, b_z: rows 2..
+    tma_load_3d(buf + L::OWX, &m->sv, bar, tl.y - 4 + EFWI_GX, tl.z, a.vf);            // forward v_x, v_z: rows 2..
+    tma_load_3d(buf + L::OLAM, &m->mc, bar, tl.y + EFWI_GX, tl.z + 2, 0);      // lambda, mu, mu_xz: tile
+    tma_load_3d(buf + L::OG, &m->gi, bar, tl.y + EFWI_GX, tl.z + 2, 0);        // imaging sums: tile
 }
 
 // A 2-byte snapshot element as a float (the conversion of the per-thread-load kernels).

@@ -60,12 +60,12 @@ __device__ __forceinline__ void issue_fwd(const TmaFwdArgs &a, const int4 tl, fl
     // element x = cell i + GX (halo-4 column 0 = cell i0 - 4), row y = cell j + GZ: halo-4 row r
     // of the tile is map row j0 - 4 + r + GZ = tl.z - 2 + r
     const int f = 5 * a.scur;
-    tma_load_3d(buf + L::OVX, &m->s2, bar, tl.y, tl.z, f);          // vx, vz: rows 2..
-    tma_load_3d(buf + L::OSXX, &m->s1, bar, tl.y, tl.z, f + 2);     // sigma_xx: rows 2..
-    tma_load_3d(buf + L::OSZZ, &m->s3, bar, tl.y, tl.z - 1, f + 3); // sigma_zz: rows 1..
-    tma_load_3d(buf + L::OSXZ, &m->s3, bar, tl.y, tl.z - 2, f + 4); // sigma_xz: rows 0..
-    tma_load_3d(buf + L::OBX, &m->mb, bar, tl.y, tl.z, 3);          // b_x, b_z: rows 2..
-    tma_load_3d(buf + L::OLAM, &m->mc, bar, tl.y + 4, tl.z + 2, 0); // lambda, mu, mu_xz: tile
+    tma_load_3d(buf + L::OVX, &m->s2, bar, tl.y - 4 + EFWI_GX, tl.z, f);          // vx, vz: rows 2..
+    tma_load_3d(buf + L::OSXX, &m->s1, bar, tl.y - 4 + EFWI_GX, tl.z, f + 2);     // sigma_xx: rows 2..
+    tma_load_3d(buf + L::OSZZ, &m->s3, bar, tl.y - 4 + EFWI_GX, tl.z - 1, f + 3); // sigma_zz: rows 1..
+    tma_load_3d(buf + L::OSXZ, &m->s3, bar, tl.y - 4 + EFWI_GX, tl.z - 2, f + 4); // sigma_xz: rows 0..
+    tma_load_3d(buf + L::OBX, &m->mb, bar, tl.y - 4 + EFWI_GX, tl.z, 3);          // b_x, b_z: rows 2..
+    tma_load_3d(buf + L::OLAM, &m->mc, bar, tl.y + EFWI_GX, tl.z + 2, 0); // lambda, mu, mu_xz: tile
 }
 
 // The arguments of a forward step of plan p (k_tma.cu).

@@ -316,10 +316,10 @@ __global__ void __launch_bounds__(kThreads, TX * TZ <= 512 ? 4 : 2) k_adj_fused(
             if (a.pf && tid == 0 && t + (int)gridDim.x < a.ntiles) {
                 // the next tile's inputs into L2 while this one computes
                 const AdjMaps *mp = a.maps + tl_next.x;
-                tma_prefetch_3d(&mp->ad, tl_next.y, tl_next.z - 2, a.acur5);
-                tma_prefetch_3d(&mp->m5, tl_next.y, tl_next.z - 2, 0);
-                if (a.sgf >= 0) tma_prefetch_3d(&mp->sg, tl_next.y, tl_next.z - 2, a.sgf);
-                tma_prefetch_3d(&mp->gi, tl_next.y + 4, tl_next.z + 2, 0);
+                tma_prefetch_3d(&mp->ad, tl_next.y - 4 + EFWI_GX, tl_next.z - 2, a.acur5);
+                tma_prefetch_3d(&mp->m5, tl_next.y - 4 + EFWI_GX, tl_next.z - 2, 0);
+                if (a.sgf >= 0) tma_prefetch_3d(&mp->sg, tl_next.y - 4 + EFWI_GX, tl_next.z - 2, a.sgf);
+                tma_prefetch_3d(&mp->gi, tl_next.y + EFWI_GX, tl_next.z + 2, 0);
             }
             __syncthreads();
 

@@ -33,12 +33,12 @@ constexpr int kThreads = 256;
 __device__ __forceinline__ void prefetch_fwd(const TmaFwdArgs &a, int4 tl) {
     const FwdMaps *m = a.maps + tl.x;
     const int f = 5 * a.scur;
-    tma_prefetch_3d(&m->s2, tl.y, tl.z, f);
-    tma_prefetch_3d(&m->s1, tl.y, tl.z, f + 2);
-    tma_prefetch_3d(&m->s3, tl.y, tl.z - 1, f + 3);
-    tma_prefetch_3d(&m->s3, tl.y, tl.z - 2, f + 4);
-    tma_prefetch_3d(&m->mb, tl.y, tl.z, 3);
-    tma_prefetch_3d(&m->mc, tl.y + 4, tl.z + 2, 0);
+    tma_prefetch_3d(&m->s2, tl.y - 4 + EFWI_GX, tl.z, f);
+    tma_prefetch_3d(&m->s1, tl.y - 4 + EFWI_GX, tl.z, f + 2);
+    tma_prefetch_3d(&m->s3, tl.y - 4 + EFWI_GX, tl.z - 1, f + 3);
+    tma_prefetch_3d(&m->s3, tl.y - 4 + EFWI_GX, tl.z - 2, f + 4);
+    tma_prefetch_3d(&m->mb, tl.y - 4 + EFWI_GX, tl.z, 3);
+    tma_prefetch_3d(&m->mc, tl.y + EFWI_GX, tl.z + 2, 0);
 }
 
 // Shared-memory output staging (ST = 1, cell pairs only): the new stresses of the
@@ -779,9 +779,9 @@ __device__ __forceinline__ void issue_adj(const TmaAdjArgs &a, int t, float *buf
     const int4 tl = a.tiles[t];
     const AdjMaps *m = a.maps + tl.x;
     mbar_expect_tx(bar, L::BYTES);
-    tma_load_3d(buf, &m->ad, bar, tl.y, tl.z - 2, 5 * a.acur);
-    tma_load_3d(buf + 5 * L::NS, &m->m5, bar, tl.y, tl.z - 2, 0);
-    tma_load_3d(buf + 10 * L::NS, &m->sg, bar, tl.y, tl.z - 2, 2 * a.slot);
+    tma_load_3d(buf, &m->ad, bar, tl.y - 4 + EFWI_GX, tl.z - 2, 5 * a.acur);
+    tma_load_3d(buf + 5 * L::NS, &m->m5, bar, tl.y - 4 + EFWI_GX, tl.z - 2, 0);
+    tma_load_3d(buf + 10 * L::NS, &m->sg, bar, tl.y - 4 + EFWI_GX, tl.z - 2, 2 * a.slot);
 }
 
 template <int TX, int TZ, int NST>
