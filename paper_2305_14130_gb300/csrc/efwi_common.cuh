@@ -6,11 +6,14 @@
 //   Each field of shot s is a block of (NZ + 2*GZ) rows x pitch floats; cell
 //   (i, j) of the padded grid sits at  off_s + (j + GZ) * pitch + (i + GX).
 //   GX = 4 left ghost columns keep every row's first interior cell 16-byte
-//   aligned (float4); pitch = roundup(NX, 8) + 8 leaves >= 4 zero columns on
-//   the right and keeps rows of 2-byte snapshot elements 16-byte aligned too
-//   (tensor copies); GZ = 2 zero rows above and below.  Ghost cells are zero and
-//   never written, so the radius-2 staggered stencils need no bounds checks
-//   and the discrete derivative operators are exact transposes up to sign.
+//   aligned (float4); a tile's halo box starts at element i0 - 4 + GX of a row,
+//   which tensor copies of 2-byte snapshot elements need at a multiple of 8 (tiles
+//   start at multiples of 32 columns: GX = 4 modulo 8); pitch =
+//   roundup(NX + 8, 32) leaves >= 4 zero columns on the right and starts every
+//   row, and so every halo box, on a 128-byte line; GZ = 2 zero rows above and
+//   below.  Ghost cells are zero and never written, so the radius-2 staggered
+//   stencils need no bounds checks and the discrete derivative operators are exact
+//   transposes up to sign.
 //   Field kinds (vx, vz, sxx, szz, sxz, materials, adjoint fields, imaging
 //   accumulators) are separate arrays sharing the per-shot offsets off_s.
 //
@@ -35,8 +38,9 @@
 #define EFWI_FLAG_SELFTEST 4     // the timeout self-test's wait expired (as intended)
 #define EFWI_FLAG_SHEAR 8        // a gradient call met mu <= 0 (or lambda + mu <= 0, scaled-stress adjoint)
 
-#define EFWI_GX 8
+#define EFWI_GX 4
 #define EFWI_GZ 2
+static_assert(EFWI_GX % 8 == 4, "halo boxes of 2-byte elements start at a multiple of 16 bytes");
 
 namespace efwi {
 
