@@ -764,10 +764,13 @@ int efwi_autotune(efwi_plan *p) {
     // (reproducible profiles, tests of one layout)
     const char *fs = getenv("EFWI_TMA_STAGES"), *fv = getenv("EFWI_TMA_VEC");
     const int only_nst = fs ? atoi(fs) : 0, only_vec = fv ? atoi(fv) : 0;
+    // EFWI_PREFETCH=0|1 forces the L2 prefetch (below) off or on; on, it keeps the layouts that have one
+    const char *fe = getenv("EFWI_PREFETCH");
+    const int force_pf = fe ? atoi(fe) : -1;
     for (auto &s : kShapes) {
         if (fixed && (s.tx != p->tile_x || s.tz != p->tile_z)) continue;
         if (want == EFWI_STENCIL_AUTO || want == EFWI_STENCIL_LOADS) fwd.push_back({EFWI_STENCIL_LOADS, s.tx, s.tz, 0});
-        for (int vec = 1; vec <= (tile_ok(p) ? 5 : 3); ++vec)
+        for (int vec = 1; vec <= (tile_ok(p) && force_pf <= 0 ? 5 : 3); ++vec)
             for (int stg = 0; stg <= 1; ++stg) {
                 const int kind = vec == 1 ? EFWI_STENCIL_TMA : stg ? EFWI_STENCIL_TMA_STAGED : EFWI_STENCIL_TMA_PAIRS;
                 if (want != EFWI_STENCIL_AUTO && want != kind) continue;
@@ -876,11 +879,9 @@ int efwi_autotune(efwi_plan *p) {
     rc = select_fwd(p, bf);
     if (!rc) rc = select_adj(p, ba);
     // L2 prefetch one tile beyond what the chosen forward (TMA) and adjoint (persistent
-    // per-thread loads) steps load: kept when it saves more than 1 %.  EFWI_PREFETCH=0|1
-    // forces it off or on (reproducible profiles and tests of one variant).
+    // per-thread loads) steps load: kept when it saves more than 1 %, or as
+    // EFWI_PREFETCH says (reproducible profiles and tests of one variant).
     {
-        const char *fe = getenv("EFWI_PREFETCH");
-        const int force_pf = fe ? atoi(fe) : -1;
         p->tma_pf = p->adj_pf = 0;
         const bool fwd_ok = !rc && p->stencil >= EFWI_STENCIL_TMA && p->tma_vec < 4;
         const bool adj_ok = !rc && p->adj_stencil == EFWI_STENCIL_LOADS && p->adj_grid > 0 &&
