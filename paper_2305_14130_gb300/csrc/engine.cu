@@ -188,7 +188,7 @@ void adjoint_loop(efwi_plan *p, cudaStream_t st) {
     cudaMemsetAsync(p->G, 0, sizeof(float) * 5 * F, st);
     if (p->Gtot) cudaMemsetAsync(p->Gtot, 0, sizeof(float) * 5 * F, st);
     if (p->Gcmp) cudaMemsetAsync(p->Gcmp, 0, sizeof(float) * 5 * F, st);
-    if (p->d.ntr > 0) cudaMemsetAsync(p->tr_acc, 0, sizeof(double) * p->d.ntr, st);
+    launch_das_adj_scan(p, st);
     p->acur = 0;
     p->apsi_v = 0;
     p->apsi_s = 0;

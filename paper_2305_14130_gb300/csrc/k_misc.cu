@@ -145,29 +145,42 @@ __global__ void k_das_fwd(const ShotDev *shots, const int *tr_shot, const int *t
     d[(long long)t * nt + n] = out;
 }
 
-// Adjoint source of step n: coefficient of trace t (reverse cumulative residual for strain).
-__global__ void k_das_adj_prep(const float *resid, double *acc, float *coef, int t0, int ntr, int nt, int n, float dt,
-                               int strain) {
-    const int t = t0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= t0 + ntr) return;
-    const float r = resid[(long long)t * nt + n];
-    if (strain) {
-        const double a = acc[t] + r;
-        acc[t] = a;
-        coef[t] = (float)((double)dt * a);
-    } else {
-        coef[t] = r;
+// Adjoint-source coefficients of every step from the residual, in place: strain-rate data take the
+// residual itself; strain data dt times its reverse running sum in FP64 (K_r^T of the time integral).
+// The sums are one serial FP64 chain per trace, so a warp takes 32 traces and brings 32 steps of each
+// through shared memory at a time.  It runs once per gradient; a launch per step in its place cost
+// 1.3 us a step (200 x 100, one shot: 19.4 -> 18.1 ms per gradient of 1000 steps).
+constexpr int kScan = 32;
+__global__ void __launch_bounds__(kScan) k_das_adj_scan(float *resid, int ntr, int nt, float dt) {
+    __shared__ float sh[kScan][kScan + 1];
+    const int lane = threadIdx.x, t0 = blockIdx.x * kScan, rows = min(kScan, ntr - t0);
+    double acc = 0.0;
+    for (int n0 = (nt - 1) / kScan * kScan; n0 >= 0; n0 -= kScan) {
+        const int cols = min(kScan, nt - n0);
+        float *r = resid + (long long)t0 * nt + n0;
+        for (int k = 0; k < rows; ++k)
+            if (lane < cols) sh[k][lane] = r[(long long)k * nt + lane];
+        __syncwarp();
+        if (lane < rows)
+            for (int n = cols - 1; n >= 0; --n) {
+                acc = acc + sh[lane][n];
+                sh[lane][n] = (float)((double)dt * acc);
+            }
+        __syncwarp();
+        for (int k = 0; k < rows; ++k)
+            if (lane < cols) r[(long long)k * nt + lane] = sh[k][lane];
+        __syncwarp();
     }
 }
 
 // Transposed sampling as a deterministic gather over the cells touched by gauge
 // ends; also the b-imaging contribution of this adjoint increment.
-__global__ void k_das_adj_gather(const ShotDev *shots, GatherCSR g, const float *coef, Fields A, const float *vfx,
+__global__ void k_das_adj_gather(const ShotDev *shots, GatherCSR g, const float *coef, int nt, Fields A, const float *vfx,
                                  const float *vfz, SnapR sr, float *Gbx, float *Gbz, int g0, int gn) {
     const int k = g0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= g0 + gn) return;
     float inc = 0.f;
-    for (int e = g.ptr[k]; e < g.ptr[k + 1]; ++e) inc += g.w[e] * coef[g.tr[e]];
+    for (int e = g.ptr[k]; e < g.ptr[k + 1]; ++e) inc += g.w[e] * coef[(long long)g.tr[e] * nt];   // coef: the step's column
     const int shot = g.tgt_shot[k];
     const long long c = shots[shot].off + g.tgt_off[k];
     if (g.tgt_field[k] == 0) {
@@ -439,19 +452,19 @@ void launch_das_fwd(efwi_plan *p, Fields F, int n, float *d, int shot, cudaStrea
     p->launches++;
 }
 
+void launch_das_adj_scan(efwi_plan *p, cudaStream_t st) {
+    if (p->d.ntr == 0 || p->d.das_mode != EFWI_DAS_STRAIN) return;
+    k_das_adj_scan<<<(p->d.ntr + kScan - 1) / kScan, kScan, 0, st>>>(p->resid, p->d.ntr, p->d.nt, (float)p->d.dt);
+    p->launches++;
+}
+
 void launch_das_adj(efwi_plan *p, Fields A, const SnapIn &si, float *Gbx, float *Gbz, int n, int shot,
                     cudaStream_t st) {
-    const int t0 = shot < 0 ? 0 : p->shots[shot].tr0;
-    const int cnt = shot < 0 ? p->d.ntr : p->shots[shot].ntr;
-    if (cnt == 0) return;
-    k_das_adj_prep<<<(cnt + 127) / 128, 128, 0, st>>>(p->resid, p->tr_acc, p->tr_coef, t0, cnt, p->d.nt, n,
-                                                      (float)p->d.dt, p->d.das_mode == EFWI_DAS_STRAIN);
     const int g0 = shot < 0 ? 0 : p->gather_ptr[shot];
     const int gn = shot < 0 ? p->gather.n_tgt : p->gather_ptr[shot + 1] - p->gather_ptr[shot];
-    p->launches++;
     if (gn == 0) return;
-    k_das_adj_gather<<<(gn + 127) / 128, 128, 0, st>>>(p->shots_d, p->gather, p->tr_coef, A, si.fx, si.fz, si.sr,
-                                                       Gbx, Gbz, g0, gn);
+    k_das_adj_gather<<<(gn + 127) / 128, 128, 0, st>>>(p->shots_d, p->gather, p->resid + n, p->d.nt, A, si.fx, si.fz,
+                                                       si.sr, Gbx, Gbz, g0, gn);
     p->launches++;
 }
 

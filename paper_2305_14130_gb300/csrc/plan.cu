@@ -284,7 +284,7 @@ static void commit_acq(efwi_plan *p, const AcqHost &h) {
 static void free_plan(efwi_plan *p) {
     if (!p) return;
     void *ptrs[] = {p->shots_d, p->state[0], p->mat, p->adj[0], p->fwd_maps, p->adj_maps, p->adjs_maps, p->dev_err, p->tile_count, p->G, p->Gtot, p->Gcmp, p->psi, p->apsi,
-                    p->prof, p->dw, p->wv, p->ref, p->tr_shot, p->tr_off, p->tr_w, p->tr_acc, p->tr_coef,
+                    p->prof, p->dw, p->wv, p->ref, p->tr_shot, p->tr_off, p->tr_w, p->tr_acc,
                     p->gather.tgt_shot, p->gather.tgt_field, p->gather.tgt_off, p->gather.ptr, p->gather.tr,
                     p->gather.w, p->tiles.tiles, p->adj_tiles.tiles, p->resid, p->dbuf, p->partial, p->seg, p->ck.fields, p->ck.psi,
                     p->ck.scale, p->segh, p->segmax, p->zoi_b, p->zoi_bp, p->zoi_sink};
@@ -479,7 +479,6 @@ extern "C" int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *d) {
     A(&p->tr_off, h_off.size(), "trace offsets");
     A(&p->tr_w, h_w.size(), "trace weights");
     A(&p->tr_acc, (size_t)std::max(ntr, 1), "trace accumulators");
-    A(&p->tr_coef, (size_t)std::max(ntr, 1), "trace coefficients");
     if (p->gather.n_tgt > 0) {
         A(&p->gather.tgt_shot, g_shot.size(), "gather");
         A(&p->gather.tgt_field, g_field.size(), "gather");

@@ -100,14 +100,13 @@ struct efwi_plan {
     int *tr_shot = nullptr;                // [ntr]
     int *tr_off = nullptr;                 // [ntr][16] offsets within shot block
     float *tr_w = nullptr;                 // [ntr][16] weights * (+-t) / L
-    double *tr_acc = nullptr;              // [ntr] running strain (fwd) / reverse residual sum (adj)
-    float *tr_coef = nullptr;              // [ntr] adjoint-source coefficient of the current step
+    double *tr_acc = nullptr;              // [ntr] running strain of the forward pass
     efwi::GatherCSR gather;
     std::vector<int> gather_ptr;           // [ns+1] per-shot range of gather targets
     int gather_nnz = 0;                    // (trace, weight) entries of the gather
     efwi::TileList tiles;                  // forward fused-step work items
     efwi::TileList adj_tiles;              // adjoint fused-step work items
-    float *resid = nullptr;                // [ntr][nt]
+    float *resid = nullptr;                // [ntr][nt] residual, then the adjoint-source coefficients
     float *dbuf = nullptr;                 // [ntr][nt]
     double *partial = nullptr;             // reduction scratch
     // Snapshot slots, one per kept step v^{n+1/2} (x and z planes): slots 0 .. K-1 hold the
@@ -182,6 +181,8 @@ void launch_materials(efwi_plan *p, const float *vp, const float *vs, const floa
 void launch_inject(efwi_plan *p, Fields F, int n, int shot /* -1 = all */, cudaStream_t st);
 void launch_force(efwi_plan *p, Fields F, int n, int shot, float *segx, float *segz, cudaStream_t st);
 void launch_das_fwd(efwi_plan *p, Fields F, int n, float *d, int shot, cudaStream_t st);
+// the residual becomes the adjoint-source coefficients of every step (once per gradient)
+void launch_das_adj_scan(efwi_plan *p, cudaStream_t st);
 void launch_das_adj(efwi_plan *p, Fields A, const SnapIn &si, float *Gbx, float *Gbz, int n, int shot,
                     cudaStream_t st);
 // packs v of state buffer scur (the last step of a pass) into the snapshot slot sw.h with maxima sw.hmax
