@@ -79,7 +79,8 @@ void clear_snap_max(efwi_plan *p, int k0, int k1, cudaStream_t st) {
         cudaMemsetAsync(efwi::snap_max(p, k0), 0, sizeof(float) * (size_t)(k1 - k0) * 2 * p->d.ns * kMaxPad, st);
 }
 
-// One forward step of every shot; d == nullptr skips the DAS sampling.
+// One forward step of every shot; d == nullptr skips the DAS sampling (else the caller steps through
+// n = 0 .. nt-1).
 void forward_step(efwi_plan *p, int n, float *d, const SnapOut &so, cudaStream_t st) {
     if (p->d.exec == EFWI_EXEC_PLAIN) {
         Fields F = state_fields(p, 0);
@@ -91,8 +92,11 @@ void forward_step(efwi_plan *p, int n, float *d, const SnapOut &so, cudaStream_t
             launch_inject(p, F, n, s, st);
         }
     } else {
-        launch_step_fused(p, n, so, st);       // leaves v^{n+1/2}, sigma^{n+1} in state[scur]
-        if (d) launch_das_fwd(p, state_fields(p, p->scur), n, d, -1, st);
+        // v^{n+1/2}, sigma^{n+1} stay in state[scur] until step n + 2 overwrites them, so step n + 1
+        // can sample the traces of step n where its kernel does that: a launch less per step
+        const bool late = d && step_samples_das(p);
+        launch_step_fused(p, n, so, st, late && n > 0 ? d : nullptr);
+        if (d && (!late || n == p->d.nt - 1)) launch_das_fwd(p, state_fields(p, p->scur), n, d, -1, st);
     }
 }
 

@@ -2,6 +2,7 @@
 // of a staged tile and its copies.
 #pragma once
 
+#include "das.cuh"
 #include "plan.hpp"
 #include "tma.cuh"
 
@@ -26,6 +27,8 @@ struct TmaFwdArgs {
     int ofield;                 // state-map field of the written buffer's vx (output staging)
     int segf;                   // segment-map field of this step's vx, or -1 (output staging)
     SnapW sw;                   // reduced-precision snapshot work (sw.h / sw.amax null: none)
+    DasArgs das;                // lean kernel: traces of the previous step to sample (das.d null: none),
+    int ncta, das0, das_ctas;   // CTAs with tiles; first CTA that samples and how many do
     int pf;                     // 1: L2 prefetch of the tile one beyond the shared-memory pipeline
 };
 
@@ -69,6 +72,6 @@ __device__ __forceinline__ void issue_fwd(const TmaFwdArgs &a, const int4 tl, fl
 }
 
 // The arguments of a forward step of plan p (k_tma.cu).
-TmaFwdArgs tma_fwd_args(efwi_plan *p, int n, const SnapOut &so);
+TmaFwdArgs tma_fwd_args(efwi_plan *p, int n, const SnapOut &so);   // das empty
 
 }  // namespace efwi

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_tile(TmaAdjsArgs a, float m
     TileFeed feed;
     if (tid == kIssue) {
         issue_adjs<kTX, kTZ, SK>(a, tl, smb, &bar[0]);
-        if (DYN) feed.start(a.tiles, a.ntiles, a.count);
+        if (DYN) feed.start((int)gridDim.x, a.tiles, a.ntiles, a.count);
     }
     // halo-4 position of the thread's pair of the tile or of the velocity ring
     const bool own = tid < kOwn, ring = !own && tid - kOwn < kRing;
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_tile(TmaAdjsArgs a, float m
             __syncthreads();
             if (DYN) {
                 tl_next = next_s;
-                if (tid == kIssue) feed.advance(a.tiles, a.ntiles, a.count);
+                if (tid == kIssue) feed.advance((int)gridDim.x, a.tiles, a.ntiles, a.count);
             }
 
             // 3. F += dt C (-D^T e^) on the tile, with the imaging in F

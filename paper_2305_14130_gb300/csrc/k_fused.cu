@@ -644,11 +644,11 @@ AdjArgsF adj_args_f(efwi_plan *p, const SnapIn &si) {
     return a;
 }
 
-void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st) {
+void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st, float *d_prev) {
     int slot;
     prof_begin(p, st, &slot, EFWI_KERNEL_STEP);
     if (p->stencil >= EFWI_STENCIL_TMA) {
-        launch_step_tma(p, n, so, st);
+        launch_step_tma(p, n, so, d_prev, st);
     } else {
         FwdArgs a = fwd_args(p, n, so);
         const int grid = p->grid_fwd_override > 0 ? std::min(p->grid_fwd_override, a.ntiles) : a.ntiles;

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "das.cuh"
 #include "plan.hpp"
 #include "reg_block.cuh"
 
@@ -120,29 +121,10 @@ __global__ void k_force(const ShotDev *shots, Fields F, Mat M, const float *wv, 
         }
 }
 
-// --------------------------------------------------------------------------
-// DAS sampling K_r (eq. 3): strain rate of trace t = sum of 16 weighted
-// velocity samples (weights carry +-t_k / L); strain = running time integral.
-// --------------------------------------------------------------------------
-__global__ void k_das_fwd(const ShotDev *shots, const int *tr_shot, const int *tr_off, const float *tr_w,
-                          double *acc, const float *vx, const float *vz, float *d, int t0, int ntr, int nt, int n,
-                          float dt, int strain) {
-    const int t = t0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= t0 + ntr) return;
-    const long long base = shots[tr_shot[t]].off;
-    float rate = 0.f;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const float *f = (k >> 2) & 1 ? vz : vx;
-        rate += tr_w[t * 16 + k] * f[base + tr_off[t * 16 + k]];
-    }
-    float out = rate;
-    if (strain) {
-        const double a = acc[t] + (double)dt * rate;
-        acc[t] = a;
-        out = (float)a;
-    }
-    d[(long long)t * nt + n] = out;
+// DAS sampling K_r (das.cuh).
+__global__ void k_das_fwd(const ShotDev *shots, DasArgs a) {
+    const int t = a.t0 + blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < a.t0 + a.ntr) das_sample(shots, a, t);
 }
 
 // Adjoint-source coefficients of every step from the residual, in place: strain-rate data take the
@@ -447,8 +429,10 @@ void launch_das_fwd(efwi_plan *p, Fields F, int n, float *d, int shot, cudaStrea
     const int t0 = shot < 0 ? 0 : p->shots[shot].tr0;
     const int cnt = shot < 0 ? p->d.ntr : p->shots[shot].ntr;
     if (cnt == 0) return;
-    k_das_fwd<<<(cnt + 127) / 128, 128, 0, st>>>(p->shots_d, p->tr_shot, p->tr_off, p->tr_w, p->tr_acc, F.vx, F.vz, d,
-                                                 t0, cnt, p->d.nt, n, (float)p->d.dt, p->d.das_mode == EFWI_DAS_STRAIN);
+    DasArgs a = das_args(p, F, n, d);
+    a.t0 = t0;
+    a.ntr = cnt;
+    k_das_fwd<<<(cnt + 127) / 128, 128, 0, st>>>(p->shots_d, a);
     p->launches++;
 }
 

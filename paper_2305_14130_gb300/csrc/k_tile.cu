@@ -34,6 +34,14 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
     __shared__ int4 next_s;
     __shared__ unsigned wmax_s[2 * (kThreads / 32)];
     const int tid = threadIdx.x;
+    auto sample = [&]() {                        // this CTA's share of the previous step's traces
+        for (int k = ((int)blockIdx.x - a.das0) * kThreads + tid; k < a.das.ntr; k += a.das_ctas * kThreads)
+            das_sample(a.shots, a.das, k);
+    };
+    if ((int)blockIdx.x >= a.ncta) {
+        sample();
+        return;
+    }
     const PairOps op{make_float2(mz, mz)};
     if (tid == 0) {
         for (int b = 0; b < kNST; ++b) mbar_init(&bar[b], 1);
@@ -44,8 +52,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
     TileFeed feed;
     if (tid == kIssue) {
         issue_fwd<kTX, kTZ, kNST, 2>(a, tl, smb, &bar[0]);
-        if (DYN) feed.start(a.tiles, a.ntiles, a.count);
+        if (DYN) feed.start(a.ncta, a.tiles, a.ntiles, a.count);
     }
+    if (a.das.d && (int)blockIdx.x >= a.das0) sample();
     // this thread's pair of the tile (16 pairs a row) and, on the first 104 threads, its pair of the
     // ring around it (rows -2, -1, 16, 17 over 18 pairs, then one pair left and right of each row)
     const int px = 2 * (tid & 15), py = tid >> 4;
@@ -64,7 +73,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
     const float2 dt2 = PairOps::both(a.dt), rx2 = PairOps::both(a.rdx), rz2 = PairOps::both(a.rdz);
     uint32_t phase = 0;
     int b = 0;
-    int t = blockIdx.x + gridDim.x;              // the next tile (at a stride)
+    int t = blockIdx.x + a.ncta;              // the next tile (at a stride)
     for (;; b ^= 1) {
         float *buf = smb + b * L::BUF;
         const ShotDev *sp = a.shots + tl.x;
@@ -194,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
             __syncthreads();
             if (DYN) {
                 tl_next = next_s;
-                if (tid == kIssue) feed.advance(a.tiles, a.ntiles, a.count);
+                if (tid == kIssue) feed.advance(a.ncta, a.tiles, a.ntiles, a.count);
             }
             if (SNAP && a.sw.amax && tid == 32) snap_max_commit(wmax_s, a.sw.amax, tl.x, a.sw.ns);
 
@@ -266,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
             return;
         }
         tl = tl_next;
-        t += gridDim.x;
+        t += a.ncta;
         if (tl.x < 0) break;
     }
 }
@@ -298,9 +307,25 @@ int tile_blocks_per_sm(int sk, int vec) {
     return std::max(1, nb);
 }
 
-void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st) {
-    const TmaFwdArgs a = tma_fwd_args(p, n, so);
-    const int grid = std::min(p->grid_fwd_override > 0 ? p->grid_fwd_override : p->tma_grid, a.ntiles);
+void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cudaStream_t st) {
+    TmaFwdArgs a = tma_fwd_args(p, n, so);
+    a.ncta = std::min(p->grid_fwd_override > 0 ? p->grid_fwd_override : p->tma_grid, a.ntiles);
+    int grid = a.ncta;
+    if (d_prev && p->d.ntr > 0) {
+        // CTAs of their own for the traces where all fit on the device at once (on a CTA with tiles
+        // the sampling's two dependent loads would lengthen the step); else the last CTAs take them
+        // before their tiles.  A launch after the step cost 2 us: 1000 x 300, 32 shots, 300 steps
+        // 43.3 -> 42.4 ms, 128 x 128, 4 shots, gradient 13.5 -> 11.6 ms
+        a.das = das_args(p, state_fields(p, p->scur), n - 1, d_prev);
+        a.das_ctas = (p->d.ntr + kThreads - 1) / kThreads;
+        if (grid + a.das_ctas <= p->tma_grid) {
+            a.das0 = a.ncta;
+            grid += a.das_ctas;
+        } else {
+            a.das_ctas = std::min(a.das_ctas, a.ncta);
+            a.das0 = a.ncta - a.das_ctas;
+        }
+    }
     with_variant(p->snap_store, p->tma_vec == 4, [&](auto k, auto d) {
         k_step_tile<decltype(k)::value, decltype(d)::value><<<grid, kThreads, L::smem(), st>>>(a, -0.f);
     });

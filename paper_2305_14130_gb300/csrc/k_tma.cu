@@ -703,12 +703,14 @@ TmaFwdArgs tma_fwd_args(efwi_plan *p, int n, const SnapOut &so) {
     a.segf = segx ? (int)((segx - p->seg) / p->fsz_total) : -1;
     a.sw = so.sw;
     a.pf = p->tma_pf;
+    a.das = DasArgs{};
+    a.ncta = a.das0 = a.das_ctas = 0;
     return a;
 }
 
-void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st) {
+void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cudaStream_t st) {
     if (p->tma_vec >= 4) {
-        launch_step_tile(p, n, so, st);
+        launch_step_tile(p, n, so, d_prev, st);
         return;
     }
     const TmaFwdArgs a = tma_fwd_args(p, n, so);

@@ -55,7 +55,7 @@ __device__ __forceinline__ float *at_byte(float *base, unsigned bytes) {
 }
 
 // Tiles of a persistent grid handed out by a counter in device memory as CTAs become free (the first
-// gridDim.x statically).  With a fixed stride instead, a CTA meets only a few tile columns when the
+// ncta, their number, statically).  With a fixed stride instead, a CTA meets only a few tile columns when the
 // grid and the tiles per row share factors, and those that hold the slower CPML tiles finish last
 // (adjoint, 32 shots of 1000 x 300 with 1 CPML cell, 32 tiles per row on 304 CTAs: 292 us against
 // 194 us with the counter); where they share none the stride balances by itself and needs no work
@@ -67,8 +67,8 @@ __device__ __forceinline__ float *at_byte(float *base, unsigned bytes) {
 struct TileFeed {
     int4 next;                   // the CTA's next work item (x < 0: none)
     int q;                       // number drawn for the one after
-    __device__ __forceinline__ void draw(const int4 *tiles, int ntiles, int *count) {
-        const int t = (int)gridDim.x + q;
+    __device__ __forceinline__ void draw(int ncta, const int4 *tiles, int ntiles, int *count) {
+        const int t = ncta + q;
         if (t < ntiles) {
             next = __ldg(tiles + t);
             q = atomicAdd(count, 1);
@@ -77,13 +77,13 @@ struct TileFeed {
             next.x = -1;
         }
     }
-    __device__ __forceinline__ void start(const int4 *tiles, int ntiles, int *count) {
+    __device__ __forceinline__ void start(int ncta, const int4 *tiles, int ntiles, int *count) {
         q = atomicAdd(count, 1);
-        draw(tiles, ntiles, count);
+        draw(ncta, tiles, ntiles, count);
     }
     // the work item after `next` becomes `next`
-    __device__ __forceinline__ void advance(const int4 *tiles, int ntiles, int *count) {
-        if (next.x >= 0) draw(tiles, ntiles, count);
+    __device__ __forceinline__ void advance(int ncta, const int4 *tiles, int ntiles, int *count) {
+        if (next.x >= 0) draw(ncta, tiles, ntiles, count);
     }
 };
 

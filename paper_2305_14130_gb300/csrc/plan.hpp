@@ -217,11 +217,13 @@ void launch_adj_stress_plain(efwi_plan *p, int shot, const float *vfx, const flo
 // lean form of 3 with tiles from a counter / at a fixed stride (k_tile.cu; 32 x 16, two stages)
 bool tma_shape_ok(int tx, int tz, int nst, int vec, int st, int snap);
 int tma_prepare_fwd(efwi_plan *p, int tx, int tz, int nst, int vec, int st);
-void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st);
+void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cudaStream_t st);
 // --- k_tile.cu -----------------------------------------------------------------
 bool tile_ok(const efwi_plan *p);           // the lean kernels' 32-bit offsets reach every field element
 int tile_blocks_per_sm(int snap_store, int vec);
-void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st);
+void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cudaStream_t st);
+// the forward steps can sample the traces of the step before them
+inline bool step_samples_das(const efwi_plan *p) { return p->stencil >= EFWI_STENCIL_TMA && p->tma_vec >= 4; }
 bool tma_adj_shape_ok(int tx, int tz, int nst);
 int tma_prepare_adj(efwi_plan *p, int tx, int tz, int nst);
 int tma_encode_adj_maps(efwi_plan *p, int tx, int tz);
@@ -245,7 +247,8 @@ int adj_tile_blocks_per_sm(int snap_store, int vec);
 void launch_adj_tile(efwi_plan *p, const SnapIn &si, cudaStream_t st);
 
 // --- k_fused.cu --------------------------------------------------------------
-void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st);
+// d_prev: data whose samples of step n - 1 the step takes as well (step_samples_das; null: none)
+void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st, float *d_prev = nullptr);
 void launch_adj_fused(efwi_plan *p, int n, const SnapIn &si, cudaStream_t st);
 int upload_tiles(efwi_plan *p, TileList &tl, int tx, int tz);
 // the work items of tile list tl (same shape and order) with the flags of another acquisition
