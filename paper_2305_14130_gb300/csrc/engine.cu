@@ -260,7 +260,10 @@ int replay(efwi_plan *p, GraphCache &gc, cudaStream_t st, Body body) {
         return cuda_status(p, "stream capture query");
     }
     if (cs == cudaStreamCaptureStatusActive) {
+        // plain launches: the caller may put the capture into the body of a conditional node
+        p->chained = false;
         body(st);
+        p->chained = true;
         return cuda_status(p, "time loop inside a stream capture");
     }
     if (!gc.exec) {

@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "adjs_tile.cuh"
+#include "chain.cuh"
 #include "pair_ops.cuh"
 
 namespace efwi {
@@ -60,8 +61,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_tile(TmaAdjsArgs a, float m
         mbar_init(&bar[1], 1);
         fence_mbar_init();
     }
-    __syncthreads();
     int4 tl = __ldg(a.tiles + blockIdx.x);       // the grid has at most ntiles CTAs
+    __syncthreads();
+    chain_begin();
     TileFeed feed;
     if (tid == kIssue) {
         issue_adjs<kTX, kTZ, SK>(a, tl, smb, &bar[0]);
@@ -364,7 +366,7 @@ void launch_adj_tile(efwi_plan *p, const SnapIn &si, cudaStream_t st) {
     const int grid = std::min(p->grid_adj_override > 0 ? p->grid_adj_override : p->tma_adj_grid, a.ntiles);
     with_variant(p->snap_store, p->adjs_vec == 4, [&](auto k, auto d) {
         constexpr int K = decltype(k)::value;
-        k_adj_tile<K, decltype(d)::value><<<grid, kThreads, smem_bytes<K>(), st>>>(a, -0.f);
+        launch_chained(chain_adj(p), k_adj_tile<K, decltype(d)::value>, grid, kThreads, smem_bytes<K>(), st, a, -0.f);
     });
 }
 

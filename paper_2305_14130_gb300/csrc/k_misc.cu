@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "chain.cuh"
 #include "das.cuh"
 #include "plan.hpp"
 #include "reg_block.cuh"
@@ -124,6 +125,7 @@ __global__ void k_force(const ShotDev *shots, Fields F, Mat M, const float *wv, 
 // DAS sampling K_r (das.cuh).
 __global__ void k_das_fwd(const ShotDev *shots, DasArgs a) {
     const int t = a.t0 + blockIdx.x * blockDim.x + threadIdx.x;
+    chain_begin();
     if (t < a.t0 + a.ntr) das_sample(shots, a, t);
 }
 
@@ -160,6 +162,7 @@ __global__ void __launch_bounds__(kScan) k_das_adj_scan(float *resid, int ntr, i
 __global__ void k_das_adj_gather(const ShotDev *shots, GatherCSR g, const float *coef, int nt, Fields A, const float *vfx,
                                  const float *vfz, SnapR sr, float *Gbx, float *Gbz, int g0, int gn) {
     const int k = g0 + blockIdx.x * blockDim.x + threadIdx.x;
+    chain_begin();
     if (k >= g0 + gn) return;
     float inc = 0.f;
     for (int e = g.ptr[k]; e < g.ptr[k + 1]; ++e) inc += g.w[e] * coef[(long long)g.tr[e] * nt];   // coef: the step's column
@@ -432,7 +435,7 @@ void launch_das_fwd(efwi_plan *p, Fields F, int n, float *d, int shot, cudaStrea
     DasArgs a = das_args(p, F, n, d);
     a.t0 = t0;
     a.ntr = cnt;
-    k_das_fwd<<<(cnt + 127) / 128, 128, 0, st>>>(p->shots_d, a);
+    launch_chained(chain_fwd(p), k_das_fwd, (cnt + 127) / 128, 128, 0, st, p->shots_d, a);
     p->launches++;
 }
 
@@ -447,8 +450,8 @@ void launch_das_adj(efwi_plan *p, Fields A, const SnapIn &si, float *Gbx, float 
     const int g0 = shot < 0 ? 0 : p->gather_ptr[shot];
     const int gn = shot < 0 ? p->gather.n_tgt : p->gather_ptr[shot + 1] - p->gather_ptr[shot];
     if (gn == 0) return;
-    k_das_adj_gather<<<(gn + 127) / 128, 128, 0, st>>>(p->shots_d, p->gather, p->resid + n, p->d.nt, A, si.fx, si.fz,
-                                                       si.sr, Gbx, Gbz, g0, gn);
+    launch_chained(chain_adj(p), k_das_adj_gather, (gn + 127) / 128, 128, 0, st, p->shots_d, p->gather, p->resid + n,
+                   p->d.nt, A, si.fx, si.fz, si.sr, Gbx, Gbz, g0, gn);
     p->launches++;
 }
 

@@ -11,6 +11,7 @@
 #include <string>
 #include <type_traits>
 
+#include "chain.cuh"
 #include "fwd_tile.cuh"
 #include "pair_ops.cuh"
 
@@ -39,6 +40,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
             das_sample(a.shots, a.das, k);
     };
     if ((int)blockIdx.x >= a.ncta) {
+        chain_begin();
         sample();
         return;
     }
@@ -47,8 +49,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
         for (int b = 0; b < kNST; ++b) mbar_init(&bar[b], 1);
         fence_mbar_init();
     }
-    __syncthreads();
     int4 tl = __ldg(a.tiles + blockIdx.x);       // the grid has at most ntiles CTAs
+    __syncthreads();
+    chain_begin();
     TileFeed feed;
     if (tid == kIssue) {
         issue_fwd<kTX, kTZ, kNST, 2>(a, tl, smb, &bar[0]);
@@ -327,7 +330,7 @@ void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cud
         }
     }
     with_variant(p->snap_store, p->tma_vec == 4, [&](auto k, auto d) {
-        k_step_tile<decltype(k)::value, decltype(d)::value><<<grid, kThreads, L::smem(), st>>>(a, -0.f);
+        launch_chained(chain_fwd(p), k_step_tile<decltype(k)::value, decltype(d)::value>, grid, kThreads, L::smem(), st, a, -0.f);
     });
 }
 

@@ -159,6 +159,7 @@ struct efwi_plan {
     bool seg_double = false;               // segment buffer holds two halves (overlap)
     efwi::GraphCache g_fwd, g_fwd_ck, g_adj, g_ph;
     bool use_graphs = true;
+    bool chained = true;                   // time-loop kernels may overlap their start with the launch before (chain.cuh)
 
     // timing of the dominant kernels (event pairs, tagged by kernel kind)
     int prof_every = 0;
