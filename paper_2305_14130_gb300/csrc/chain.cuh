@@ -19,7 +19,7 @@ namespace efwi {
 // and the waiting CTAs take the places of the last tiles' CTAs: 1000 x 300, 32 shots, 300 steps
 // 42.3 -> 42.8 ms; 8 shots with the energy sum between the steps 15.5 -> 16.0 ms.
 inline bool chain_fwd(const efwi_plan *p) {
-    return p->chained && step_samples_das(p) && p->tiles.n <= p->tma_grid;
+    return p->chained && lean_fwd(p) && p->tiles.n <= p->tma_grid;
 }
 inline bool chain_adj(const efwi_plan *p) {
     return p->chained && p->adj_form == EFWI_ADJ_FORM_SCALED && p->adj_stencil == EFWI_STENCIL_TMA &&

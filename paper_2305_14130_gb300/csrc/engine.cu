@@ -94,8 +94,8 @@ void forward_step(efwi_plan *p, int n, float *d, const SnapOut &so, cudaStream_t
     } else {
         // v^{n+1/2}, sigma^{n+1} stay in state[scur] until step n + 2 overwrites them, so step n + 1
         // can sample the traces of step n where its kernel does that: a launch less per step
-        const bool late = d && step_samples_das(p);
-        launch_step_fused(p, n, so, st, late && n > 0 ? d : nullptr);
+        const bool late = d && lean_fwd(p);
+        launch_step_fused(p, n, so, st, StepMore{late && n > 0 ? d : nullptr});
         if (d && (!late || n == p->d.nt - 1)) launch_das_fwd(p, state_fields(p, p->scur), n, d, -1, st);
     }
 }
@@ -385,6 +385,10 @@ extern "C" int efwi_pseudo_hessian(efwi_plan *p, const float *vp, const float *v
         reset_forward_state(p, cs);
         cudaMemsetAsync(acc, 0, sizeof(float) * 2 * p->fsz_total, cs);
         for (int n = 0; n < p->d.nt; ++n) {
+            if (p->d.exec == EFWI_EXEC_BATCHED && lean_fwd(p)) {
+                launch_step_fused(p, n, SnapOut{}, cs, StepMore{nullptr, acc, cmp});
+                continue;
+            }
             forward_step(p, n, nullptr, SnapOut{}, cs);
             launch_vel_energy(p, state_fields(p, p->d.exec == EFWI_EXEC_PLAIN ? 0 : p->scur), acc, cmp, cs);
         }

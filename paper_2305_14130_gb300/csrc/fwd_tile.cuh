@@ -29,6 +29,7 @@ struct TmaFwdArgs {
     SnapW sw;                   // reduced-precision snapshot work (sw.h / sw.amax null: none)
     DasArgs das;                // lean kernel: traces of the previous step to sample (das.d null: none),
     int ncta, das0, das_ctas;   // CTAs with tiles; first CTA that samples and how many do
+    float *esum, *ecmp;         // lean kernel: |v|^2 of the step goes to this compensated sum (null: not)
     int pf;                     // 1: L2 prefetch of the tile one beyond the shared-memory pipeline
 };
 

@@ -644,11 +644,11 @@ AdjArgsF adj_args_f(efwi_plan *p, const SnapIn &si) {
     return a;
 }
 
-void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st, float *d_prev) {
+void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st, const StepMore &more) {
     int slot;
     prof_begin(p, st, &slot, EFWI_KERNEL_STEP);
     if (p->stencil >= EFWI_STENCIL_TMA) {
-        launch_step_tma(p, n, so, d_prev, st);
+        launch_step_tma(p, n, so, more, st);
     } else {
         FwdArgs a = fwd_args(p, n, so);
         const int grid = p->grid_fwd_override > 0 ? std::min(p->grid_fwd_override, a.ntiles) : a.ntiles;
@@ -715,8 +715,8 @@ float time_steps(efwi_plan *p, bool adj, cudaStream_t st, cudaEvent_t e0, cudaEv
             if (adj) {
                 launch_adj_fused(p, 0, si, st);
             } else {
-                const bool late = das && step_samples_das(p);
-                launch_step_fused(p, n, so, st, late ? p->dbuf : nullptr);
+                const bool late = das && lean_fwd(p);
+                launch_step_fused(p, n, so, st, StepMore{late ? p->dbuf : nullptr});
                 if (das && !late) launch_das_fwd(p, state_fields(p, p->scur), n, p->dbuf, -1, st);
             }
         }

@@ -25,7 +25,10 @@ constexpr int kIssue = 224;                      // the thread that issues the c
 constexpr int kRingRow = kTX / 2 + 2, kRing = 4 * kRingRow + 2 * kTZ;   // cell pairs of the velocity halo ring
 
 // DYN: tiles from the counter (TileFeed), else at a stride of the grid
-template <int SK, bool DYN>
+// EN: the pseudo-Hessian's sum of |v|^2 (k_hessian.cu's expressions on the staged v^{n+1/2}).  A pass
+// of its own reads v from memory again and costs a launch per step: 8 shots of 1000 x 300, 300 steps
+// 15.4 -> 14.4 ms.
+template <int SK, bool DYN, bool EN = false>
 __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float mz) {
     constexpr bool SNAP = SK != 0;
     extern __shared__ float4 smem_raw[];
@@ -214,6 +217,39 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
             if (!edge || ncell > 0) {
                 const float *svx = buf + L::OVX - 2 * kSX + so, *svz = buf + L::OVZ - 2 * kSX + so;
                 const float2 vb = ld2(svx), wb = ld2(svz);
+                if constexpr (EN) {
+                    bool phys[2] = {true, true};
+                    if (edge) {
+                        const int P = __ldg(&sp->P), i = tl.y + px, j = tl.z + py;
+                        const bool row = j >= P && j < __ldg(&sp->NZ) - P;
+                        for (int h = 0; h < 2; ++h) phys[h] = row && i + h >= P && i + h < __ldg(&sp->NX) - P;
+                    }
+                    float *es = at_byte(a.esum, 4u * c0), *ec = at_byte(a.ecmp, 4u * c0);
+                    float2 sum = make_float2(0.f, 0.f), cmp = sum;
+                    if (!edge || (phys[0] && phys[1])) {
+                        sum = ld2(es);
+                        cmp = ld2(ec);
+                    } else {
+                        if (phys[0]) { sum.x = es[0]; cmp.x = ec[0]; }
+                        if (phys[1]) { sum.y = es[1]; cmp.y = ec[1]; }
+                    }
+                    const float2 wu = ld2(svz - kSX);
+                    auto add = [&](float &s, float &c, float v0, float v1, float w0, float w1) {
+                        const float vx = 0.5f * (v0 + v1), vz = 0.5f * (w0 + w1);
+                        const float y = (vx * vx + vz * vz) - c, t1 = s + y;
+                        c = (t1 - s) - y;
+                        s = t1;
+                    };
+                    add(sum.x, cmp.x, svx[-1], vb.x, wu.x, wb.x);
+                    add(sum.y, cmp.y, vb.x, vb.y, wu.y, wb.y);
+                    if (!edge || (phys[0] && phys[1])) {
+                        st2(es, sum);
+                        st2(ec, cmp);
+                    } else {
+                        if (phys[0]) { es[0] = sum.x; ec[0] = cmp.x; }
+                        if (phys[1]) { es[1] = sum.y; ec[1] = cmp.y; }
+                    }
+                }
                 float2 f1 = op.mul(op.diff_m(ld2(svx - 2), vb, svx[2]), rx2);
                 float2 f2 = op.mul(op.diff(wb, ld2(svz - kSX), ld2(svz + kSX), ld2(svz - 2 * kSX)), rz2);
                 float2 f3 = op.mul(op.diff(ld2(svx + kSX), vb, ld2(svx + 2 * kSX), ld2(svx - kSX)), rz2);
@@ -305,21 +341,24 @@ int tile_blocks_per_sm(int sk, int vec) {
         constexpr auto kernel = k_step_tile<decltype(k)::value, decltype(d)::value>;
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::smem());
         cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        constexpr auto energy = k_step_tile<0, decltype(d)::value, true>;
+        cudaFuncSetAttribute(energy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::smem());
+        cudaFuncSetAttribute(energy, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kThreads, L::smem());
     });
     return std::max(1, nb);
 }
 
-void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cudaStream_t st) {
+void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, const StepMore &more, cudaStream_t st) {
     TmaFwdArgs a = tma_fwd_args(p, n, so);
     a.ncta = std::min(p->grid_fwd_override > 0 ? p->grid_fwd_override : p->tma_grid, a.ntiles);
     int grid = a.ncta;
-    if (d_prev && p->d.ntr > 0) {
+    if (more.d_prev && p->d.ntr > 0) {
         // CTAs of their own for the traces where all fit on the device at once (on a CTA with tiles
         // the sampling's two dependent loads would lengthen the step); else the last CTAs take them
         // before their tiles.  A launch after the step cost 2 us: 1000 x 300, 32 shots, 300 steps
         // 43.3 -> 42.4 ms, 128 x 128, 4 shots, gradient 13.5 -> 11.6 ms
-        a.das = das_args(p, state_fields(p, p->scur), n - 1, d_prev);
+        a.das = das_args(p, state_fields(p, p->scur), n - 1, more.d_prev);
         a.das_ctas = (p->d.ntr + kThreads - 1) / kThreads;
         if (grid + a.das_ctas <= p->tma_grid) {
             a.das0 = a.ncta;
@@ -328,6 +367,14 @@ void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cud
             a.das_ctas = std::min(a.das_ctas, a.ncta);
             a.das0 = a.ncta - a.das_ctas;
         }
+    }
+    if (more.esum) {
+        a.esum = more.esum;
+        a.ecmp = more.ecmp;
+        with_variant(EFWI_STORE_FP32, p->tma_vec == 4, [&](auto k, auto d) {
+            launch_chained(chain_fwd(p), k_step_tile<0, decltype(d)::value, true>, grid, kThreads, L::smem(), st, a, -0.f);
+        });
+        return;
     }
     with_variant(p->snap_store, p->tma_vec == 4, [&](auto k, auto d) {
         launch_chained(chain_fwd(p), k_step_tile<decltype(k)::value, decltype(d)::value>, grid, kThreads, L::smem(), st, a, -0.f);

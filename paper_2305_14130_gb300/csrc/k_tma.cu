@@ -704,13 +704,14 @@ TmaFwdArgs tma_fwd_args(efwi_plan *p, int n, const SnapOut &so) {
     a.sw = so.sw;
     a.pf = p->tma_pf;
     a.das = DasArgs{};
+    a.esum = a.ecmp = nullptr;
     a.ncta = a.das0 = a.das_ctas = 0;
     return a;
 }
 
-void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cudaStream_t st) {
+void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, const StepMore &more, cudaStream_t st) {
     if (p->tma_vec >= 4) {
-        launch_step_tile(p, n, so, d_prev, st);
+        launch_step_tile(p, n, so, more, st);
         return;
     }
     const TmaFwdArgs a = tma_fwd_args(p, n, so);

@@ -218,13 +218,18 @@ void launch_adj_stress_plain(efwi_plan *p, int shot, const float *vfx, const flo
 // lean form of 3 with tiles from a counter / at a fixed stride (k_tile.cu; 32 x 16, two stages)
 bool tma_shape_ok(int tx, int tz, int nst, int vec, int st, int snap);
 int tma_prepare_fwd(efwi_plan *p, int tx, int tz, int nst, int vec, int st);
-void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cudaStream_t st);
+// What a lean forward step can take along (lean_fwd; null pointers: nothing).
+struct StepMore {
+    float *d_prev = nullptr;                   // data whose samples of step n - 1 it takes
+    float *esum = nullptr, *ecmp = nullptr;    // compensated sum of |v|^2 that it adds step n to
+};
+void launch_step_tma(efwi_plan *p, int n, const SnapOut &so, const StepMore &more, cudaStream_t st);
 // --- k_tile.cu -----------------------------------------------------------------
 bool tile_ok(const efwi_plan *p);           // the lean kernels' 32-bit offsets reach every field element
 int tile_blocks_per_sm(int snap_store, int vec);
-void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, float *d_prev, cudaStream_t st);
-// the forward steps can sample the traces of the step before them
-inline bool step_samples_das(const efwi_plan *p) { return p->stencil >= EFWI_STENCIL_TMA && p->tma_vec >= 4; }
+void launch_step_tile(efwi_plan *p, int n, const SnapOut &so, const StepMore &more, cudaStream_t st);
+// the forward steps are lean ones: they can take the work of StepMore along
+inline bool lean_fwd(const efwi_plan *p) { return p->stencil >= EFWI_STENCIL_TMA && p->tma_vec >= 4; }
 bool tma_adj_shape_ok(int tx, int tz, int nst);
 int tma_prepare_adj(efwi_plan *p, int tx, int tz, int nst);
 int tma_encode_adj_maps(efwi_plan *p, int tx, int tz);
@@ -248,8 +253,7 @@ int adj_tile_blocks_per_sm(int snap_store, int vec);
 void launch_adj_tile(efwi_plan *p, const SnapIn &si, cudaStream_t st);
 
 // --- k_fused.cu --------------------------------------------------------------
-// d_prev: data whose samples of step n - 1 the step takes as well (step_samples_das; null: none)
-void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st, float *d_prev = nullptr);
+void launch_step_fused(efwi_plan *p, int n, const SnapOut &so, cudaStream_t st, const StepMore &more = StepMore{});
 void launch_adj_fused(efwi_plan *p, int n, const SnapIn &si, cudaStream_t st);
 int upload_tiles(efwi_plan *p, TileList &tl, int tx, int tz);
 // the work items of tile list tl (same shape and order) with the flags of another acquisition

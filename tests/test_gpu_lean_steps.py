@@ -63,3 +63,21 @@ def test_lean_step_windows_sources_and_snapshots(efwi, monkeypatch, source, snap
     for layout in (4, 5):
         for a, b in zip(_run(efwi, monkeypatch, p, layout, **kw), ref):
             assert torch.equal(a, b), layout
+
+
+# the step's own sum of |v|^2 and the pass that follows a step of the kernels that load per thread
+@pytest.mark.parametrize("nx,nz,win", [(52, 36, None), (51, 35, None), (53, 37, None),
+                                       (170, 45, [[20, 90], [13, 157], [0, 170]])])
+def test_lean_step_sums_the_energy(efwi, monkeypatch, nx, nz, win):
+    p = rounded(W.tiny(nx=nx, nz=nz, ns=3, nt=36, npml=5, win=win))
+    out = []
+    for layout in (0, 4, 5):
+        if layout:
+            monkeypatch.setenv("EFWI_TMA_VEC", str(layout))
+        plan = efwi.Plan(p.acq, exec="batched", stencil="tma_pairs" if layout else "loads", tile=(32, 16))
+        assert not layout or plan.info()["layout"] == layout
+        out.append(plan.pseudo_hessian(dev(p.vp), dev(p.vs), dev(p.rho), eps=0.02))
+        plan.sync_status()
+        plan.close()
+    for h, hi in out[1:]:
+        assert torch.equal(h, out[0][0]) and torch.equal(hi, out[0][1])
