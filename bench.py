@@ -256,10 +256,13 @@ def roofline(exec_, info, prof, nt, ns):
                        4: "TMA, cell pairs, staged stores"}.get(kind, "?")
             if k == "step" and kind >= 2 and info["layout"] == 3:
                 staging += ", halo ring as single cells"
+            if k == "step" and kind >= 2 and info["layout"] >= 4:
+                staging += {4: ", packed, tiles from a counter", 5: ", packed"}[info["layout"]]
             if k == "adj" and kind == 1 and info["adj_persistent"]:
                 staging += ", persistent grid"
             if k == "adj" and kind == 2 and info.get("adj_layout", 0) >= 2:
-                staging += ", cell pairs" + (", 512 threads" if info["adj_layout"] == 3 else "")
+                staging += ", cell pairs" + {3: ", 512 threads", 4: ", packed, tiles from a counter",
+                                              5: ", packed"}.get(info["adj_layout"], "")
             if k == "adj" and info.get("adj_form", 1) == 2:
                 staging = "scaled-stress form, " + staging
             name = f"{name.split(' ')[0]} [{staging}, tile {tile[0]}x{tile[1]}] {' '.join(name.split(' ')[1:])}"

@@ -8,12 +8,12 @@
 // component (vx at i -+ 1/2, vz at j -+ 1/2), and the clipped, scaled inverse
 //   P(x) = c / max(H(x), c),  c = eps * max_x H   (P = 1 everywhere if H = 0).
 //
-// k_vel_energy runs after every forward step (the lean one, k_tile.cu, does the same work itself) and adds |v|^2 of every physical
-// node of every shot, in FP32, to a Kahan-compensated FP32 sum with the
-// wavefield layout (the same precision as the imaging sums); k_ph_collect adds
-// the compensated sums of the shots covering each physical pixel in FP64
-// (fixed shot order) and takes block maxima; k_max_final and k_ph_scale finish
-// the inverse.
+// k_vel_energy runs after every forward step (the lean one, k_tile.cu, does the
+// same work itself) and adds |v|^2 of every physical node of every shot, in
+// FP32, to a Kahan-compensated FP32 sum with the wavefield layout (the same
+// precision as the imaging sums); k_ph_collect adds the compensated sums of the
+// shots covering each physical pixel in FP64 (fixed shot order) and takes block
+// maxima; k_max_final and k_ph_scale finish the inverse.
 #include <algorithm>
 
 #include "plan.hpp"

@@ -7,6 +7,12 @@
 //     accesses are one base and constants, its global ones one 32-bit offset;
 //   * the CPML memory of an edge tile loaded before the wait for the tile's copies, all of it in
 //     flight together, instead of in each half step after the barrier.
+// The cell-pair kernel issued about 300 instructions a cell and was bound by their latencies.  32 shots
+// of 1000 x 300, keeping v: 176 -> 163 us (68 B a cell without CPML memory: 4.8 TB/s, 70 % of the
+// measured HBM bandwidth; copies and stores of 60 B alone, without arithmetic, take 115 us); FP16 snapshots, 8 shots 53 -> 47 us;
+// 200 x 100, one shot, with the sampling 8.8 -> 4.8 us, where the chain of a tile's copies, two
+// barriers and stores is what is left.  Tried and slower: 64 x 16 tiles in 512 threads, three stages
+// with the moduli in registers (195 us), a CTA marching down a strip with its rows in registers (165 to 190 us).
 #include <algorithm>
 #include <string>
 #include <type_traits>
