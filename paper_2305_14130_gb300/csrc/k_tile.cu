@@ -1,13 +1,14 @@
 // Forward time step with TMA staging, lean form of k_tma.cu's split cell-pair layout: the same
 // persistent grid, 32 x 16 tiles, stages and copies, and the same arithmetic, term by term (all
-// variants agree bit for bit), with far fewer instructions per cell:
+// variants agree bit for bit), with fewer instructions and waits per cell:
 //   * packed FP32 arithmetic on a thread's cell pair (PairOps);
 //   * the halo ring of the velocity region as 104 cell pairs instead of 208 single cells;
 //   * every position of a thread inside a tile computed once per launch: a tile's shared-memory
 //     accesses are one base and constants, its global ones one 32-bit offset;
 //   * the CPML memory of an edge tile loaded before the wait for the tile's copies, all of it in
 //     flight together, instead of in each half step after the barrier.
-// The cell-pair kernel issued about 300 instructions a cell and was bound by their latencies.  32 shots
+// The cell-pair kernel was bound by its warps' barriers and load latencies at 260 instructions a cell
+// (205 now; barrier 3.2 and long-scoreboard 2.3 of 10 stalls per instruction are what is left).  32 shots
 // of 1000 x 300, keeping v: 176 -> 163 us (68 B a cell without CPML memory: 4.8 TB/s, 70 % of the
 // measured HBM bandwidth; copies and stores of 60 B alone, without arithmetic, take 115 us); FP16 snapshots, 8 shots 53 -> 47 us;
 // 200 x 100, one shot, with the sampling 8.8 -> 4.8 us, where the chain of a tile's copies, two
