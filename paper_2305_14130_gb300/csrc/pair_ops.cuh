@@ -59,7 +59,7 @@ __device__ __forceinline__ float *at_byte(float *base, unsigned bytes) {
 // grid and the tiles per row share factors, and those that hold the slower CPML tiles finish last
 // (adjoint, 32 shots of 1000 x 300 with 1 CPML cell, 32 tiles per row on 304 CTAs: 292 us against
 // 194 us with the counter); where they share none the stride balances by itself and needs no work
-// item through shared memory (20 CPML cells, 33 tiles per row: 240 us against 250 us).  The lean
+// item through shared memory (20 CPML cells, 33 tiles per row: 247 us against 261 us).  The lean
 // kernels are compiled for both and the autotuner times them.  One thread of the CTA owns the feed;
 // the counter is read two tiles ahead and the work item one tile ahead, so neither latency is waited
 // for.  Every CTA draws exactly one number past the end; the last of these leaves the counter at zero
