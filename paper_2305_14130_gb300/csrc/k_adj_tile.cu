@@ -133,7 +133,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_tile(TmaAdjsArgs a, float m
             if (!ok_s) return false;
             mbar_wait_bounded(&bar[b], (phase >> b) & 1u);   // completed: acquire for every thread
             phase ^= 1u << b;
-            // refill the stage of the previous tile: every thread has passed the barrier above
+            // refill the stage of the previous tile: every thread has released it and passed the
+            // barrier above
             if (tid == kIssue) {
                 if (DYN) next_s = tl_next = feed.next;   // read by every thread after the next barrier
                 if (tl_next.x >= 0) issue_adjs<kTX, kTZ, SK>(a, tl_next, smb + (b ^ 1) * L::BUF, &bar[b ^ 1]);
@@ -332,6 +333,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_tile(TmaAdjsArgs a, float m
             }
             return;
         }
+        stage_release();
         tl = tl_next;
         t += gridDim.x;
         if (tl.x < 0) break;

@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(NT, 2) k_adj_scaled_tma(TmaAdjsArgs a) {
         mbar_wait_bounded(&bar[b], (phase >> b) & 1u);   // completed: acquire for every thread
         phase ^= 1u << b;
         // refill the other stage with the CTA's next tile: every thread has passed the barrier
-        // above, so none still reads that stage (it held the previous tile)
+        // above and has released that stage (it held the previous tile)
         if (tid == 0 && t + (int)gridDim.x < a.ntiles) {
             issue_adjs<TX, TZ, SK>(a, tl_fill, smb + (b ^ 1) * L::BUF, &bar[b ^ 1]);   // tile t + gridDim.x
             if (t + 2 * (int)gridDim.x < a.ntiles) tl_fill = __ldg(a.tiles + t + 2 * gridDim.x);
@@ -426,6 +426,7 @@ __global__ void __launch_bounds__(NT, 2) k_adj_scaled_tma(TmaAdjsArgs a) {
         };
         if (tl.w & 4) tile(std::true_type{});
         else tile(std::false_type{});
+        stage_release();
     }
 }
 

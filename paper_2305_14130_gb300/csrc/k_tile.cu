@@ -119,7 +119,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
             if (!ok_s) return false;
             mbar_wait_bounded(&bar[b], (phase >> b) & 1u);   // completed: acquire for every thread
             phase ^= 1u << b;
-            // refill the stage of the previous tile: every thread has passed the barrier above
+            // refill the stage of the previous tile: every thread has released it and passed the
+            // barrier above
             if (tid == kIssue) {
                 if (DYN) next_s = tl_next = feed.next;   // read by every thread after the next barrier
                 if (tl_next.x >= 0) issue_fwd<kTX, kTZ, kNST, 2>(a, tl_next, smb + (b ^ 1) * L::BUF, &bar[b ^ 1]);
@@ -320,6 +321,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tile(TmaFwdArgs a, float m
             }
             return;
         }
+        stage_release();
         tl = tl_next;
         t += a.ncta;
         if (tl.x < 0) break;

@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tma(TmaFwdArgs a) {
         mbar_wait_bounded(&bar[b], (phase >> b) & 1u);   // completed: acquire for every thread
         phase ^= 1u << b;
         // refill the stage consumed in the previous iteration with tile k + NST - 1: every
-        // thread has passed the barrier above, so none still reads that stage
+        // thread has released that stage and passed the barrier above
         const int tn = t + (NST - 1) * gridDim.x;
         const int bn = (k + NST - 1) % NST;
         if (tid == 0) {
@@ -426,7 +426,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tma(TmaFwdArgs a) {
                         oxx[c] = nxx[0]; ozz[c] = nzz[0]; oxz[c] = nxz[0];
                     }
                 }
-                if (ST) fence_proxy_async_smem();   // the staged outputs are read by bulk copies
             } else {
             // v^{n+1/2} on the tile + 2-cell halo, in place over v^{n-1/2}
                 constexpr int VX = TX + 4, VZ = TZ + 4;
@@ -551,6 +550,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_step_tma(TmaFwdArgs a) {
         };
         if (tl.w & 2) tile(std::true_type{});
         else tile(std::false_type{});
+        stage_release();                    // with ST also for the bulk stores that read the staged outputs
     }
     if (ST) {
         __syncthreads();                    // every thread has staged the last tile's outputs
@@ -996,6 +996,7 @@ __global__ void __launch_bounds__(256) k_adj_tma(TmaAdjArgs a) {
             a.out.sxz[off + c] = sxz - (C1 * (e2s[o + SX] - e2s[o]) + C2 * (e2s[o + 2 * SX] - e2s[o - SX])) * rdz
                                      - (C1 * (hvz[o + 1] - hvz[o]) + C2 * (hvz[o + 2] - hvz[o - 1])) * rdx;
         }
+        stage_release();
         __syncthreads();
     }
 }

@@ -148,4 +148,10 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// Hand a stage over to the copies that refill it: a tile's half steps store into its stage in place
+// (generic proxy), and the refill writes the same addresses through the async proxy.  A CTA barrier
+// orders generic accesses only, so every thread calls this after its last access to the stage and
+// before the barrier that the refill is issued behind.
+__device__ __forceinline__ void stage_release() { fence_proxy_async_smem(); }
+
 }  // namespace efwi
