@@ -61,6 +61,7 @@ void reset_forward_state(efwi_plan *p, cudaStream_t st) {
         if (p->state[k]) cudaMemsetAsync(p->state[k], 0, sizeof(float) * 5 * p->fsz_total, st);
     cudaMemsetAsync(p->psi, 0, sizeof(float) * 4 * p->H, st);
     if (p->d.ntr > 0) cudaMemsetAsync(p->tr_acc, 0, sizeof(double) * p->d.ntr, st);
+    cudaMemsetAsync(p->tile_count, 0, sizeof(int), st);
     p->scur = 0;
     p->psi_v = 0;
     p->psi_s = 0;
@@ -189,6 +190,7 @@ void adjoint_loop(efwi_plan *p, cudaStream_t st) {
     for (int k = 0; k < 2; ++k)
         if (p->adj[k]) cudaMemsetAsync(p->adj[k], 0, sizeof(float) * 5 * F, st);
     cudaMemsetAsync(p->apsi, 0, sizeof(float) * 4 * p->H, st);
+    cudaMemsetAsync(p->tile_count, 0, 2 * sizeof(int), st);   // the recompute's and the adjoint's
     cudaMemsetAsync(p->G, 0, sizeof(float) * 5 * F, st);
     if (p->Gtot) cudaMemsetAsync(p->Gtot, 0, sizeof(float) * 5 * F, st);
     if (p->Gcmp) cudaMemsetAsync(p->Gcmp, 0, sizeof(float) * 5 * F, st);

@@ -697,6 +697,15 @@ struct Variant {
     int kind, tx, tz, nst, vec = 1, st = 0;
 };
 
+// A wait that expired while variants were timed: a copy may have stalled, so nothing more is timed and
+// the plan is not created (efwi_sync_status, on the same flag, ends a plan).
+bool tune_timeout(efwi_plan *p) {
+    int flag = 0;
+    cudaMemcpy(&flag, p->dev_err, sizeof(int), cudaMemcpyDeviceToHost);
+    if (flag & EFWI_FLAG_TIMEOUT) p->broken = true;
+    return p->broken;
+}
+
 // time of one step in ms (adj 0: a forward step with its DAS sampling, as the data passes run it)
 float time_steps(efwi_plan *p, bool adj, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int reps = 3) {
     // the snapshot traffic of a real step: FP32 copy of v into slot 0, or the
@@ -706,6 +715,10 @@ float time_steps(efwi_plan *p, bool adj, cudaStream_t st, cudaEvent_t e0, cudaEv
     const bool das = p->d.ntr > 0 && p->d.nt > 1;
     const int n = das ? 1 : 0;
     float t = 0;
+    if (p->broken) return 1e30f;
+    // EFWI_TEST_TUNE_TIMEOUT=1: a bounded wait runs out while a variant is timed
+    const char *ft = getenv("EFWI_TEST_TUNE_TIMEOUT");
+    if (ft && ft[0] == '1') launch_selftest_timeout(p, 1 << 21, EFWI_FLAG_TIMEOUT, st);
     for (int w = 0; w < 2; ++w) {              // warm-up, then timed
         // three steps of a small grid are shorter than the start of the first one varies (200 x 100, one
         // shot: 1000 steps of 5.9 ms +- 15 % with the layouts so chosen, 4.7 ms with 24 steps timed)
@@ -724,7 +737,7 @@ float time_steps(efwi_plan *p, bool adj, cudaStream_t st, cudaEvent_t e0, cudaEv
         cudaEventSynchronize(e1);
         cudaEventElapsedTime(&t, e0, e1);
     }
-    return cudaGetLastError() == cudaSuccess ? t / reps : 1e30f;
+    return cudaGetLastError() == cudaSuccess && !tune_timeout(p) ? t / reps : 1e30f;
 }
 
 int select_adj(efwi_plan *p, const Variant &v) {
@@ -964,6 +977,7 @@ int efwi_autotune(efwi_plan *p) {
         const bool tma_adj = p->adj_stencil == EFWI_STENCIL_TMA;
         auto run = [&](int of, int oa) {
             float t = 0;
+            if (p->broken) return 1e30f;
             for (int w = 0; w < 2; ++w) {
                 cudaEventRecord(e0, sa);
                 cudaStreamWaitEvent(sr, e0);
@@ -983,7 +997,7 @@ int efwi_autotune(efwi_plan *p) {
                 cudaEventSynchronize(e1);
                 cudaEventElapsedTime(&t, e0, e1);
             }
-            return cudaGetLastError() == cudaSuccess ? t : 1e30f;
+            return cudaGetLastError() == cudaSuccess && !tune_timeout(p) ? t : 1e30f;
         };
         (void)tma_adj;
         const bool force = p->d.overlap == EFWI_OVERLAP_ON;
@@ -1029,6 +1043,7 @@ int efwi_autotune(efwi_plan *p) {
     cudaMemset(p->G, 0, sizeof(float) * 5 * p->fsz_total);
     if (p->seg) cudaMemset(p->seg, 0, sizeof(float) * (size_t)p->nslots * 2 * p->fsz_total);
     cudaMemset(p->dev_err, 0, sizeof(int));
+    cudaMemset(p->tile_count, 0, 2 * sizeof(int));
     p->scur = p->acur = p->psi_v = p->psi_s = p->apsi_v = p->apsi_s = 0;
     p->launches = 0;
     p->prof_counter[0] = p->prof_counter[1] = 0;
@@ -1037,6 +1052,10 @@ int efwi_autotune(efwi_plan *p) {
     if (e != cudaSuccess) {
         p->err = std::string("autotune: ") + cudaGetErrorString(e);
         return EFWI_ERR_CUDA;
+    }
+    if (p->broken) {
+        p->err = "autotune: a kernel gave up a bounded wait while variants were timed";
+        return EFWI_ERR_TIMEOUT;
     }
     if (rc && p->err.empty()) p->err = "autotune: could not prepare the selected variant";
     return rc;

@@ -1096,20 +1096,30 @@ void launch_adj_tma(efwi_plan *p, const float *vfx, cudaStream_t st) {
 // Self-test of the timeout path: one thread waits, with the bounded wait of the
 // TMA kernels, on an mbarrier that expects two arrivals and receives one, so
 // the phase never completes; after `budget` clock cycles the wait gives up and
-// the plan's device flag records it, exactly as a stalled copy would.  Nothing
-// else is issued (no copy, no trap), so the kernel always ends.
+// the plan's device flag records it and the tile counters stay where a CTA that
+// gave up may leave them (past their last number, not brought back to zero), as a
+// stalled copy would.  Nothing else is issued (no copy, no trap), so the kernel
+// always ends.
 // ===========================================================================
 namespace {
 
-__global__ void k_selftest_timeout(long long budget, int *err) {
+__global__ void k_selftest_timeout(long long budget, int *err, int flag, int *count) {
     __shared__ __align__(8) uint64_t bar;
     efwi::mbar_init(&bar, 2);
     efwi::fence_mbar_init();
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(efwi::smem_u32(&bar)) : "memory");
-    if (!efwi::mbar_wait_bounded(&bar, 0u, budget)) atomicOr(err, EFWI_FLAG_SELFTEST);
+    if (!efwi::mbar_wait_bounded(&bar, 0u, budget)) {
+        atomicOr(err, flag);
+        count[0] += 1 << 20;
+        count[1] += 1 << 20;
+    }
 }
 
 }  // namespace
+
+void efwi::launch_selftest_timeout(efwi_plan *p, long long budget, int flag, cudaStream_t st) {
+    k_selftest_timeout<<<1, 1, 0, st>>>(budget, p->dev_err, flag, p->tile_count);
+}
 
 extern "C" int efwi_selftest_timeout(efwi_plan *p, long long budget_cycles, efwi_stream_t stream) {
     if (!p || budget_cycles < 1 || budget_cycles > (1LL << 32)) {
@@ -1117,7 +1127,7 @@ extern "C" int efwi_selftest_timeout(efwi_plan *p, long long budget_cycles, efwi
         if (p) p->err = "budget outside [1, 2^32] cycles";
         return EFWI_ERR_ARG;
     }
-    k_selftest_timeout<<<1, 1, 0, (cudaStream_t)stream>>>(budget_cycles, p->dev_err);
+    efwi::launch_selftest_timeout(p, budget_cycles, EFWI_FLAG_SELFTEST, (cudaStream_t)stream);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         p->err = std::string("efwi_selftest_timeout: ") + cudaGetErrorString(e);

@@ -140,7 +140,8 @@ struct efwi_plan {
                                            // 3 = cell pairs in 512-thread CTAs, 4, 5 = packed cell pairs
     int tma_adj_grid = 0, tma_adj_stages = 1;
     int adj_grid = 0;                      // per-thread-load adjoint: persistent grid (0 = one CTA per tile)
-    int *tile_count = nullptr;             // tile counters of the lean forward and adjoint steps (zero between launches)
+    int *tile_count = nullptr;             // tile counters of the lean forward and adjoint steps: zero between launches, unless a
+                                           // CTA gave up its wait; cleared at the start of every time loop
     int *dev_err = nullptr;                // device flag: a bounded wait expired
     bool broken = false;                   // a real bounded wait expired: the plan is not used again
     int adj_tile_x = 0, adj_tile_z = 0;    // adjoint tile
@@ -233,6 +234,8 @@ inline bool lean_fwd(const efwi_plan *p) { return p->stencil >= EFWI_STENCIL_TMA
 bool tma_adj_shape_ok(int tx, int tz, int nst);
 int tma_prepare_adj(efwi_plan *p, int tx, int tz, int nst);
 int tma_encode_adj_maps(efwi_plan *p, int tx, int tz);
+// a bounded wait that runs out after `budget` cycles and raises `flag`
+void launch_selftest_timeout(efwi_plan *p, long long budget, int flag, cudaStream_t st);
 void launch_adj_tma(efwi_plan *p, const float *vfx, cudaStream_t st);
 
 // --- k_adjs.cu (adjoint step in scaled-stress form) ----------------------------
