@@ -46,8 +46,10 @@ __device__ double lb_block_sum(double v) {
 // conversions and a multiply-add, at about 2 per SM and clock): 0.15 ms for 28.8 M elements whose
 // bytes take 0.034 ms.  Here a thread's 8 products of one iteration are summed in FP32 with their
 // rounding errors carried along (two-product, two-sum) after both factors are scaled by a power of
-// two to at most 1, so that no error term underflows, and only that sum is added in FP64: half an
-// FP64 operation per element, error about 2^-47 of sum |x y|.
+// two to at most 1, and only that sum is added in FP64: half an FP64 operation per element, error
+// about 2^-47 of sum |x y|.  A product below 2^-100 of the two largest factors (x large where y is
+// small and the other way round) would lose its error term to underflow: such a chunk is summed in
+// FP64 too, as is one with an infinity or NaN.
 __device__ double chunk_dot(const float (&x)[kLbChunk], const float (&y)[kLbChunk]) {
     int ex = 0, ey = 0;
 #pragma unroll
@@ -57,12 +59,7 @@ __device__ double chunk_dot(const float (&x)[kLbChunk], const float (&y)[kLbChun
     }
     ex >>= 23;
     ey >>= 23;
-    if (ex == 255 || ey == 255) {                // an infinity or NaN: the plain FP64 sum
-        double v = 0.0;
-#pragma unroll
-        for (int j = 0; j < kLbChunk; ++j) v += (double)x[j] * (double)y[j];
-        return v;
-    }
+    bool wide = ex == 255 || ey == 255;          // an infinity or NaN
     // 2^(126 - ex): the largest magnitude becomes [1/2, 1); an exponent below 1 (subnormals) is left
     // as if it were 1
     ex = max(ex, 1);
@@ -73,9 +70,16 @@ __device__ double chunk_dot(const float (&x)[kLbChunk], const float (&y)[kLbChun
     for (int j = 0; j < kLbChunk; ++j) {
         const float a = x[j] * kx, b = y[j] * ky;
         const float p = a * b, e = __fmaf_rn(a, b, -p);
+        wide |= fabsf(p) < 0x1p-100f && x[j] != 0.f && y[j] != 0.f;
         const float s = hi + p, t = s - hi;
         lo += ((hi - (s - t)) + (p - t)) + e;
         hi = s;
+    }
+    if (wide) {
+        double v = 0.0;
+#pragma unroll
+        for (int j = 0; j < kLbChunk; ++j) v += (double)x[j] * (double)y[j];
+        return v;
     }
     // 1 / (kx ky), exact in FP64
     const double un = __hiloint2double((1023 + 252 - max(253 - ex, 1) - max(253 - ey, 1) + 2) << 20, 0);
