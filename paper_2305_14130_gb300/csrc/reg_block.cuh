@@ -14,7 +14,10 @@
 // (two-sum, two-product; Knuth, Dekker), and the few FP64 operations left are per pixel:
 //   * The rows of W and omega sum to 1, so every quantity is shift-invariant: with the pivot
 //     c = m_0 the differences e_s = m_s - c are exact in FP32 for components within a factor of
-//     two of each other, and sum e, sum e^2, sum b' and sum b' e give mean, 1^T r and |r|^2.
+//     two of each other, and sum e, sum e^2, sum b' and sum b' e give mean, 1^T r and |r|^2.  The
+//     pivot's own residual is -mean, which bounds the cancellation in |r|^2 by a factor of about 2 ns.
+//     W changes a component at its sinkhole, so the pivot is one without a sinkhole at the pixel;
+//     where all have one, the FP64 sums are shifted by the mean of all components.
 //   * A component whose difference is not exact, whose values leave the range in which the
 //     products' errors are representable, or which has its sinkhole here, is added in FP64.
 // A block takes 32 pixels x 8 groups of components (128-byte rows; a grid of few pixels
@@ -82,7 +85,8 @@ struct RegSums {
 struct RegShared {
     float f[kRegGroups][8][kRegPx];
     double x[kRegGroups][3][kRegPx];
-    double B[kRegPx], BE[kRegPx], delta[kRegPx], cy[kRegPx];
+    double B[kRegPx], BE[kRegPx], h[kRegPx], delta[kRegPx], rwd[kRegPx];
+    int first[kRegGroups][kRegPx];
     float rw[kRegPx], dh[kRegPx], dl[kRegPx];
 };
 
@@ -102,7 +106,7 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
     float mv[N], bpv[N], gv[N];
     unsigned smask = 0;
     bool any = false;
-    const float c = live ? m[p] : 0.f;
+    float c = live ? m[p] : 0.f;
     if (KEEP) {
 #pragma unroll
         for (int k = 0; k < N; ++k) {
@@ -155,40 +159,52 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
         }
     };
 
-    // 1. where a sinkhole lies: B and sum b_i e_i of its pixel
+    // 1. where a sinkhole lies: the pivot, B and sum b_i e_i of its pixel
     const bool block_sink = __syncthreads_or(any && ns > 1) != 0;
+    bool pixel_sink = false;
     if (block_sink) {
+        int first = ns;                          // of the thread's components, without a sinkhole here
+        if (live)
+            for (int k = 0, s = gr; s < ns && first == ns; ++k, s += kRegGroups)
+                if (KEEP ? !((smask >> k) & 1u) : sink[s * npix + p] == 0) first = s;
+        sh.first[gr][px] = any ? -1 - first : first;
+        __syncthreads();
+        first = ns;
+        for (int q = 0; q < kRegGroups; ++q) {
+            const int f = sh.first[q][px];
+            pixel_sink |= f < 0;
+            first = min(first, f < 0 ? -1 - f : f);
+        }
+        if (pixel_sink) c = m[(first < ns ? first : 0) * npix + p];
         double vb = 0, ve = 0;
-        wide_each(~0u, [&](long long o, float ms, float, bool) {
-            const double bs = b[o];
-            vb += bs;
-            ve += bs * ((double)ms - (double)c);
-        });
+        if (pixel_sink)
+            wide_each(~0u, [&](long long o, float ms, float, bool) {
+                const double bs = b[o];
+                vb += bs;
+                ve += bs * ((double)ms - (double)c);
+            });
         sh.x[gr][0][px] = vb;
         sh.x[gr][1][px] = ve;
-        sh.x[gr][2][px] = any ? 1.0 : 0.0;
         __syncthreads();
         if (gr == 0) {
-            double B = 0, BE = 0, f = 0;
-            for (int q = 0; q < kRegGroups; ++q) { B += sh.x[q][0][px]; BE += sh.x[q][1][px]; f += sh.x[q][2][px]; }
+            double B = 0, BE = 0;
+            for (int q = 0; q < kRegGroups; ++q) { B += sh.x[q][0][px]; BE += sh.x[q][1][px]; }
             sh.B[px] = B;
             sh.BE[px] = BE;
-            sh.cy[px] = f;                       // > 0: some component has its sinkhole at this pixel
+            sh.h[px] = !COLLAPSE && pixel_sink && first == ns && B != 0 ? BE / B : 0.0;
         }
         __syncthreads();
     }
-    const double B = block_sink ? sh.B[px] : 0, BE = block_sink ? sh.BE[px] : 0;
-    const bool pixel_sink = block_sink && sh.cy[px] > 0;
-    // w = (W m)_s - c in FP64, c_s and d_s - c_s b_s
+    // w = (W m)_s - (c + h) in FP64, c_s and d_s - c_s b_s
     auto wide = [&](long long o, float ms, bool in, double &cs, double &dc) {
         const double e = (double)ms - (double)c;
         cs = 0.0;
         dc = 1.0;
         if (!in) return e;
         const double bs = b[o];
-        cs = (1.0 - bs) / (B - bs);
+        cs = (1.0 - bs) / (sh.B[px] - bs);
         dc = bs - cs * bs;
-        return dc * e + cs * BE;
+        return dc * e + cs * sh.BE[px] - sh.h[px];
     };
 
     // 2. the sums over the components
@@ -250,6 +266,7 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
                 sh.delta[px] = delta;
                 sh.dh[px] = dh;
                 sh.dl[px] = (float)(delta - (double)dh);
+                sh.rwd[px] = R / sb;
                 sh.rw[px] = (float)(R / sb);
             }
         } else {
@@ -284,7 +301,7 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
                 if (!in) return;
                 double cs, dc;
                 const double v = wide(o, ms, in, cs, dc);
-                cy += cs * ((v - delta) - (double)w * (double)rw);
+                cy += cs * ((v - delta) - (double)w * sh.rwd[px]);
             });
         sh.x[gr][0][px] = cy;
         __syncthreads();
@@ -294,7 +311,7 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
         for (int q = 0; q < kRegGroups; ++q) cy += sh.x[q][0][px];
         wide_each(~0u, [&](long long o, float ms, float w, bool in) {
             double cs, dc;
-            const double y = (wide(o, ms, in, cs, dc) - delta) - (double)w * (double)rw;
+            const double y = (wide(o, ms, in, cs, dc) - delta) - (double)w * sh.rwd[px];
             g[o] = (float)((double)g[o] + eta2 * (dc * y + (double)b[o] * cy));
         });
     } else if (KEEP) {

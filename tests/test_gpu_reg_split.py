@@ -1,0 +1,65 @@
+"""Consistency term and collapse where the sums need care: sinkholes on the first or on all components.
+Reference: the FP64 oracle."""
+import ctypes as C
+
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from common import f32, rel_l2
+from oracle import extension as X
+
+pytestmark = pytest.mark.gpu
+NZ, NX = 19, 41                                           # 779 pixels: ragged blocks of 32 to 256
+
+
+@pytest.fixture(scope="module")
+def efwi():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2305_14130_gb300 as m
+    return m
+
+
+def dev(a, dtype=np.float32):
+    return torch.tensor(np.ascontiguousarray(np.asarray(a, dtype)), device="cuda")
+
+
+def _check(efwi, m, b, bp, sink, tol_phi, tol_g=1e-6):
+    """phi, gradient (both entry points) and collapse against the oracle."""
+    plan = efwi.Plan(W.tiny(nx=NX, nz=NZ, ns=2, nt=4, npml=3).acq, exec="plain")
+    args = dev(m), dev(b), dev(bp), dev(sink, np.uint8)
+    phi_o, g_o = X.regularization(m, b, bp, sink, 0.7)
+    phi, g = plan.regularization_grad(*args, 0.7)
+    phi2, g2 = torch.empty((), dtype=torch.float64, device="cuda"), torch.zeros_like(g)
+    ptr = [C.c_void_p(t.data_ptr()) for t in (*args, phi2, g2)]
+    assert efwi.load_library().efwi_regularization_grad_noalloc(
+        len(m), NX, NZ, *ptr[:4], 0.7, *ptr[4:], C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    plan.close()
+    assert torch.equal(g, g2)
+    for v in (phi, phi2):
+        assert abs(v.item() - phi_o) <= tol_phi * phi_o
+    assert rel_l2(g.cpu().numpy(), g_o) <= tol_g
+    out = efwi.collapse(*args).cpu().numpy()
+    assert rel_l2(out, X.collapse(m, b, bp, sink)) <= 1e-6
+
+
+# the first component, or every one, has its sinkhole at a pixel and is far (D = 1000) from the others,
+# whose residual is r = 0.05: a pivot there would cost (D / r)^2 = 4e8 of the sums' 47 or 53 bits.  The
+# oracle's residuals carry 2^-53 of 3000, 7e-12 of r.
+# (Two components alone would take each other's value there.)
+@pytest.mark.parametrize("ns,sinks", [(n, k) for n in (2, 4, 8, 16, 64, 257) for k in ("first", "all") if n > 2 or k == "first"])
+def test_sinkhole_of_the_first_component(efwi, ns, sinks):
+    rng = np.random.default_rng(ns)
+    m = 3000 + 0.05 * rng.standard_normal((ns, NZ, NX))
+    b = rng.uniform(0.3, 1.0, (ns, NZ, NX))
+    m[0], b[0] = 4000.0, 1e-7
+    sink = np.zeros((ns, NZ, NX), np.uint8)
+    sink[0, :, ::2] = 1
+    if sinks == "all":
+        sink[:, :, ::2] = 1
+    b = f32(b)
+    m, bp = f32(m), np.where(sink, 0.5, b)
+    m[0, :, 1::2] = f32(3000.0)                           # no outlier where it has no sinkhole
+    _check(efwi, m, b, bp, sink, 1e-9)
