@@ -18,6 +18,8 @@
 //     pivot's own residual is -mean, which bounds the cancellation in |r|^2 by a factor of about 2 ns.
 //     W changes a component at its sinkhole, so the pivot is one without a sinkhole at the pixel;
 //     where all have one, the FP64 sums are shifted by the mean of all components.
+//   * The collapse sums b' m itself: no pivot, whose infinity or size (beside a weight of 0) would
+//     spoil the others, and no difference that gradients of either sign would round.
 //   * A component whose difference is not exact, whose values leave the range in which the
 //     products' errors are representable, or which has its sinkhole here, is added in FP64.
 // A block takes 32 pixels x 8 groups of components (128-byte rows; a grid of few pixels
@@ -79,12 +81,12 @@ __device__ __forceinline__ Df df_add(Df a, const Df &b) {
 // FP32 sums of one thread's components, and the FP64 sums of those that need FP64
 struct RegSums {
     Df s1, s2, sbe, sb;                      // sum w, w^2, b' w, b' with w = (W m)_s - c
-    double x1 = 0, x2 = 0, xbe = 0;
+    double x1 = 0, x2 = 0, xbe = 0, xb = 0;
 };
 
 struct RegShared {
     float f[kRegGroups][8][kRegPx];
-    double x[kRegGroups][3][kRegPx];
+    double x[kRegGroups][4][kRegPx];
     double B[kRegPx], BE[kRegPx], h[kRegPx], delta[kRegPx], rwd[kRegPx];
     int first[kRegGroups][kRegPx];
     float rw[kRegPx], dh[kRegPx], dl[kRegPx];
@@ -106,7 +108,7 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
     float mv[N], bpv[N], gv[N];
     unsigned smask = 0;
     bool any = false;
-    float c = live ? m[p] : 0.f;
+    float c = !COLLAPSE && live ? m[p] : 0.f;
     if (KEEP) {
 #pragma unroll
         for (int k = 0; k < N; ++k) {
@@ -139,13 +141,18 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
             }
         }
     };
-    // m_s - c, and whether it and the products formed from it are safe in FP32
-    constexpr float lo_e = COLLAPSE ? 1e-25f : 1e-12f, hi_e = 1e15f;
+    // m_s - c (the collapse: m_s), and whether it and the products formed from it are safe in FP32
     auto diff = [&](float ms, float w, float &e) {
+        const float aw = fabsf(w);
+        if (COLLAPSE) {
+            e = ms;
+            const float ap = fabsf(w * ms);
+            return ((ap >= 1e-30f && ap <= 1e30f) || ms == 0.f) && aw >= 1e-12f && aw <= 1e12f;
+        }
         e = ms - c;
         const float t = e - ms, err = (ms - (e - t)) - (c + t);
         const float ae = fabsf(e);
-        return err == 0.f && (ae == 0.f || (ae >= lo_e && ae <= hi_e)) && (w == 0.f || (w >= 1e-12f && w <= 1e12f));
+        return err == 0.f && (ae == 0.f || (ae >= 1e-12f && ae <= 1e15f)) && (aw == 0.f || (aw >= 1e-12f && aw <= 1e12f));
     };
     // f(s, offset, m_s, b'_s, sinkhole flag) over the components set in a mask (with KEEP; all
     // otherwise), read again and not unrolled: the few that are added in FP64
@@ -175,7 +182,7 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
             pixel_sink |= f < 0;
             first = min(first, f < 0 ? -1 - f : f);
         }
-        if (pixel_sink) c = m[(first < ns ? first : 0) * npix + p];
+        if (!COLLAPSE && pixel_sink) c = m[(first < ns ? first : 0) * npix + p];
         double vb = 0, ve = 0;
         if (pixel_sink)
             wide_each(~0u, [&](long long o, float ms, float, bool) {
@@ -217,11 +224,12 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
         a.x1 += v;
         a.x2 += v * v;
         a.xbe += (double)w * v;
+        a.xb += w;
     };
     each([&](int k, int, long long o, float ms, float w, bool in) {
         float e;
-        a.sb.add(w);
         if (diff(ms, w, e) && !in) {
+            a.sb.add(w);
             if (!COLLAPSE) {
                 a.s1.add(e);
                 a.s2.add_product(e, e);
@@ -242,6 +250,7 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
         sh.x[gr][0][px] = a.x1;
         sh.x[gr][1][px] = a.x2;
         sh.x[gr][2][px] = a.xbe;
+        sh.x[gr][3][px] = a.xb;
         spec = true;
         __syncthreads();
     }
@@ -253,12 +262,16 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
 #pragma unroll
             for (int k = 0; k < 4; ++k) s[k].add(Df{sh.f[q][2 * k][px], sh.f[q][2 * k + 1][px]});
         if (spec) {
-            double s1 = s[0].value(), s2 = s[1].value(), sbe = s[2].value();
-            const double sb = s[3].value();
-            for (int q = 0; q < kRegGroups; ++q) { s1 += sh.x[q][0][px]; s2 += sh.x[q][1][px]; sbe += sh.x[q][2][px]; }
+            double s1 = s[0].value(), s2 = s[1].value(), sbe = s[2].value(), sb = s[3].value();
+            for (int q = 0; q < kRegGroups; ++q) {
+                s1 += sh.x[q][0][px];
+                s2 += sh.x[q][1][px];
+                sbe += sh.x[q][2][px];
+                sb += sh.x[q][3][px];
+            }
             const double delta = sbe / sb;       // mean of W m under omega, minus c
             if (COLLAPSE) {
-                if (live) out[p] = (float)((double)c + delta);
+                if (live) out[p] = (float)delta;
             } else {
                 const double R = s1 - ns * delta;                // 1^T r
                 if (live) part = s2 - delta * (s1 + R);          // sum (w - delta)^2
@@ -274,7 +287,7 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
             // the components' sums
             const Df s1 = s[0].normal(), sb = s[3].normal(), delta = df_div(s[2].normal(), sb);
             if (COLLAPSE) {
-                if (live) out[p] = df_add(Df{c, 0.f}, delta).hi;
+                if (live) out[p] = delta.hi;
             } else {
                 const Df nd = df_mul(Df{(float)-ns, 0.f}, delta), R = df_add(s1, nd), t = df_mul(delta, df_add(s1, R));
                 const Df q = df_add(s[1].normal(), Df{-t.hi, -t.lo});

@@ -1,5 +1,5 @@
-"""Consistency term and collapse where the sums need care: sinkholes on the first or on all components.
-Reference: the FP64 oracle."""
+"""Consistency term and collapse where the sums need care: sinkholes on the first or on all components,
+values that one FP32 sum does not hold.  Reference: the FP64 oracle."""
 import ctypes as C
 
 import numpy as np
@@ -24,6 +24,14 @@ def efwi():
 
 def dev(a, dtype=np.float32):
     return torch.tensor(np.ascontiguousarray(np.asarray(a, dtype)), device="cuda")
+
+
+def _weights(ns, seed, sinks=0.3):
+    rng = np.random.default_rng(seed)
+    b = f32(rng.uniform(0.05, 1.0, (ns, NZ, NX)))
+    sink = (rng.random((ns, NZ, NX)) < sinks / ns).astype(np.uint8)
+    sink[:, :7] = 0                                       # rows of pixels without any
+    return rng, b, np.where(sink, 1.0, b), sink
 
 
 def _check(efwi, m, b, bp, sink, tol_phi, tol_g=1e-6):
@@ -63,3 +71,27 @@ def test_sinkhole_of_the_first_component(efwi, ns, sinks):
     m, bp = f32(m), np.where(sink, 0.5, b)
     m[0, :, 1::2] = f32(3000.0)                           # no outlier where it has no sinkhole
     _check(efwi, m, b, bp, sink, 1e-9)
+
+
+# weights whose FP32 sum overflows; a component of weight 0 that is larger than all digits of the rest
+@pytest.mark.parametrize("ns", [2, 4, 7, 20])
+def test_collapse_of_extreme_weights_and_values(efwi, ns):
+    rng, b, bp, sink = _weights(ns, 7, sinks=0.0)
+    m = f32(rng.uniform(1500, 4000, (ns, NZ, NX)))
+    out = efwi.collapse(dev(m), dev(b), dev(bp * 3e38), dev(sink, np.uint8)).cpu().numpy()
+    assert rel_l2(out, X.collapse(m, b, np.float32(bp * 3e38).astype(np.float64), sink)) <= 1e-6
+    if ns > 2:
+        m[0], bp[0] = 1e30, 0.0
+        out = efwi.collapse(dev(m), dev(b), dev(bp), dev(sink, np.uint8)).cpu().numpy()
+        assert rel_l2(out, X.collapse(m, b, bp, sink)) <= 1e-6
+
+
+@pytest.mark.parametrize("ns", [2, 4, 7, 20])
+@pytest.mark.parametrize("s", [0, 1])
+def test_collapse_of_an_infinity(efwi, ns, s):
+    _, b, bp, sink = _weights(ns, 9, sinks=0.0)
+    m = np.full((ns, NZ, NX), 2000.0)
+    m[s, 4, 40], m[s, 11, 3] = np.inf, -np.inf
+    out = efwi.collapse(dev(m), dev(b), dev(bp), dev(sink, np.uint8)).cpu().numpy()
+    assert out[4, 40] == np.inf and out[11, 3] == -np.inf
+    assert np.isfinite(out).sum() == NZ * NX - 2
