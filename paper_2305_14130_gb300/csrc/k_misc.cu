@@ -376,24 +376,26 @@ __global__ void k_zoi(ZoiShot z, int s, int nx, int nz, double dx, double dz, do
     sink[o] = inside ? 1 : 0;
 }
 
-// Consistency term and collapse (eq. 9; eq. 15 when applied to the per-source gradients): 32
+// Consistency term and collapse (eq. 9; eq. 15 when applied to the per-source gradients): 256 / G
 // pixels per block and iteration (reg_block.cuh).
-template <int CPT>
+template <int G, int CPT>
 __global__ void __launch_bounds__(kRegThreads, reg_blocks(CPT)) k_collapse(const float *x, const float *b, const float *bp,
                                                           const uint8_t *sink, int ns, long long npix, float *out) {
     __shared__ RegShared sh;
-    for (long long p0 = (long long)blockIdx.x * kRegPx; p0 < npix; p0 += (long long)gridDim.x * kRegPx)
-        reg_block<CPT, true>(x, b, bp, sink, ns, npix, p0, 0.0, nullptr, out, sh);
+    constexpr int PX = kRegThreads / G;
+    for (long long p0 = (long long)blockIdx.x * PX; p0 < npix; p0 += (long long)gridDim.x * PX)
+        reg_block<G, CPT, true>(x, b, bp, sink, ns, npix, p0, 0.0, nullptr, out, sh);
 }
 
-template <int CPT>
+template <int G, int CPT>
 __global__ void __launch_bounds__(kRegThreads, reg_blocks(CPT)) k_reg(const float *m, const float *b, const float *bp,
                                                      const uint8_t *sink, int ns, long long npix, double eta2,
                                                      float *g, double *partial) {
     __shared__ RegShared sh;
+    constexpr int PX = kRegThreads / G;
     double acc = 0.0;
-    for (long long p0 = (long long)blockIdx.x * kRegPx; p0 < npix; p0 += (long long)gridDim.x * kRegPx)
-        acc += reg_block<CPT, false>(m, b, bp, sink, ns, npix, p0, eta2, g, nullptr, sh);
+    for (long long p0 = (long long)blockIdx.x * PX; p0 < npix; p0 += (long long)gridDim.x * PX)
+        acc += reg_block<G, CPT, false>(m, b, bp, sink, ns, npix, p0, eta2, g, nullptr, sh);
     acc = block_sum(acc);
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
@@ -566,22 +568,21 @@ int launch_zoi(int ns, int nx, int nz, double dx, double dz, const efwi_zoi_desc
     return EFWI_OK;
 }
 
-// blocks of a grid-stride pass over npix pixels: all resident at once, at most `most`
-static int reg_grid(const void *kernel, long long npix, int most) {
+// blocks of a grid-stride pass over npix pixels, px a block: all resident at once, at most `most`
+static int reg_grid(const void *kernel, int px, long long npix, int most) {
     int dev = 0, sms = 1, nb = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kRegThreads, 0);
-    return (int)std::max<long long>(1, std::min<long long>((npix + kRegPx - 1) / kRegPx,
-                                                           std::min(std::max(nb, 1) * sms, most)));
+    return (int)std::max<long long>(1, std::min<long long>((npix + px - 1) / px, std::min(std::max(nb, 1) * sms, most)));
 }
 
 void launch_collapse(int ns, long long npix, const float *x, const float *b, const float *bp, const uint8_t *sink,
                      float *out, cudaStream_t st) {
-    reg_dispatch(ns, [&](auto cpt) {
-        constexpr int C = decltype(cpt)::value;
-        const int grid = reg_grid((const void *)k_collapse<C>, npix, 1 << 16);
-        k_collapse<C><<<grid, kRegThreads, 0, st>>>(x, b, bp, sink, ns, npix, out);
+    reg_dispatch(ns, [&](auto g, auto cpt) {
+        constexpr int G = decltype(g)::value, C = decltype(cpt)::value;
+        const int grid = reg_grid((const void *)k_collapse<G, C>, kRegThreads / G, npix, 1 << 16);
+        k_collapse<G, C><<<grid, kRegThreads, 0, st>>>(x, b, bp, sink, ns, npix, out);
     });
 }
 
@@ -589,10 +590,10 @@ void launch_reg(efwi_plan *p, const float *m, const float *b, const float *bp, c
                 double *phi, float *g, int accumulate_phi, cudaStream_t st, int ns) {
     const long long npix = (long long)p->d.nz * p->d.nx;
     if (ns <= 0) ns = p->d.ns;
-    reg_dispatch(ns, [&](auto cpt) {
-        constexpr int C = decltype(cpt)::value;
-        const int grid = reg_grid((const void *)k_reg<C>, npix, kPartials);
-        k_reg<C><<<grid, kRegThreads, 0, st>>>(m, b, bp, sink, ns, npix, eta * eta, g, p->partial);
+    reg_dispatch(ns, [&](auto groups, auto cpt) {
+        constexpr int G = decltype(groups)::value, C = decltype(cpt)::value;
+        const int grid = reg_grid((const void *)k_reg<G, C>, kRegThreads / G, npix, kPartials);
+        k_reg<G, C><<<grid, kRegThreads, 0, st>>>(m, b, bp, sink, ns, npix, eta * eta, g, p->partial);
         k_final_sum<<<1, 1024, 0, st>>>(p->partial, grid, 0.5 * eta * eta, phi, accumulate_phi);
     });
     p->launches += 2;

@@ -52,14 +52,15 @@ __device__ double na_block_sum(double v) {
 }
 
 // The arithmetic of eqs. 8, 11, 12 is reg_block, the same as the plan's kernel.
-template <int CPT>
+template <int G, int CPT>
 __global__ void __launch_bounds__(kNaThreads, efwi::reg_blocks(CPT)) k_reg_noalloc(const float *m, const float *b, const float *bp,
                                                             const uint8_t *sink, int ns, long long npix, double eta2,
                                                             float *g, double *partial) {
     __shared__ efwi::RegShared sh;
+    constexpr int PX = efwi::kRegThreads / G;
     double acc = 0.0;
-    for (long long p0 = (long long)blockIdx.x * efwi::kRegPx; p0 < npix; p0 += (long long)gridDim.x * efwi::kRegPx)
-        acc += efwi::reg_block<CPT, false>(m, b, bp, sink, ns, npix, p0, eta2, g, nullptr, sh);
+    for (long long p0 = (long long)blockIdx.x * PX; p0 < npix; p0 += (long long)gridDim.x * PX)
+        acc += efwi::reg_block<G, CPT, false>(m, b, bp, sink, ns, npix, p0, eta2, g, nullptr, sh);
     acc = na_block_sum(acc);
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
@@ -139,9 +140,10 @@ extern "C" int efwi_regularization_grad_noalloc(int ns, int nx, int nz, const fl
         efwi::set_thread_error(err);
         return rc;
     }
-    const int blocks = (int)std::min<long long>((npix + efwi::kRegPx - 1) / efwi::kRegPx, kNaBlocks);
-    efwi::reg_dispatch(ns, [&](auto cpt) {
-        k_reg_noalloc<decltype(cpt)::value><<<blocks, kNaThreads, 0, st>>>(m, b, bp, sink, ns, npix, eta * eta, g,
+    const int px = efwi::kRegThreads / efwi::reg_split(ns).groups;
+    const int blocks = (int)std::min<long long>((npix + px - 1) / px, kNaBlocks);
+    efwi::reg_dispatch(ns, [&](auto groups, auto cpt) {
+        k_reg_noalloc<decltype(groups)::value, decltype(cpt)::value><<<blocks, kNaThreads, 0, st>>>(m, b, bp, sink, ns, npix, eta * eta, g,
                                                                           partial);
     });
     k_sum_noalloc<<<1, 1024, 0, st>>>(partial, blocks, 0.5 * eta * eta, phi_reg);

@@ -1,5 +1,6 @@
-"""Consistency term and collapse where the sums need care: sinkholes on the first or on all components,
-values that one FP32 sum does not hold.  Reference: the FP64 oracle."""
+"""Consistency term and collapse at the ends of every split of a pixel's components over threads, and
+where the sums need care: sinkholes on the first or on all components, values that one FP32 sum does not
+hold.  Reference: the FP64 oracle."""
 import ctypes as C
 
 import numpy as np
@@ -51,6 +52,27 @@ def _check(efwi, m, b, bp, sink, tol_phi, tol_g=1e-6):
     assert rel_l2(g.cpu().numpy(), g_o) <= tol_g
     out = efwi.collapse(*args).cpu().numpy()
     assert rel_l2(out, X.collapse(m, b, bp, sink)) <= 1e-6
+
+
+# phi: pairs of FP32 (2^-47) amplified by at most 2 ns, and the oracle's own FP64 sums
+@pytest.mark.parametrize("kind", ["near", "spread", "signed"])
+@pytest.mark.parametrize("ns", [2, 16, 17, 32, 33, 64, 65, 128, 129, 256, 257])
+def test_ends_of_the_splits(efwi, ns, kind):
+    rng, b, bp, sink = _weights(ns, 100 + ns)
+    z = rng.standard_normal((ns, NZ, NX))
+    m = {"near": 3000 + 100 * z, "spread": 10.0 ** (2 * z), "signed": 1e-9 * z * np.exp(2 * z[::-1])}[kind]
+    _check(efwi, f32(m), b, bp, sink, 1e-10)
+
+
+def test_one_component(efwi):
+    # the residual is zero, with or without a sinkhole
+    _, b, bp, sink = _weights(1, 3)
+    m = f32(np.random.default_rng(3).uniform(1500, 4000, (1, NZ, NX)))
+    plan = efwi.Plan(W.tiny(nx=NX, nz=NZ, ns=2, nt=4, npml=3).acq, exec="plain")
+    phi, g = plan.regularization_grad(dev(m), dev(b), dev(bp), dev(sink, np.uint8), 0.7)
+    assert phi.item() == 0.0 and float(g.abs().max()) == 0.0
+    assert np.array_equal(efwi.collapse(dev(m), dev(b), dev(bp), dev(sink, np.uint8)).cpu().numpy(), np.float32(m[0]))
+    plan.close()
 
 
 # the first component, or every one, has its sinkhole at a pixel and is far (D = 1000) from the others,
