@@ -23,12 +23,13 @@
 //     spoil the others, and no difference that gradients of either sign would round.
 //   * A component whose values leave the range in which the products' errors are representable,
 //     or which has its sinkhole here, is added in FP64.
-// A block takes 32 pixels x 8 groups of components (128-byte rows; a grid of few pixels still fills the
+// A block takes 256 / G pixels x G groups of components (128-byte rows; a grid of few pixels still fills the
 // chip); a thread keeps the m, b', flag and g of its components in registers, so every array is read
 // once: 17 B per component, b only where a sinkhole lies.  64 components of 2000 x 600 (1.31 GB): 1.89 ->
 // 0.79 ms, a quarter of the HBM bandwidth (1.07 ms where the differences take pairs); collapse 2.45 ->
 // 0.50 ms.  Waits for the loads of the next pixels (24 warps per SM, issue slots 40 % used) are what is
 // left.  Four blocks per SM (64 registers, spills) took 2 % longer, 16 groups of 4 kept components 19 %.
+// G falls with ns (reg_split).
 #pragma once
 
 #include <cstdint>
@@ -394,12 +395,19 @@ __device__ double reg_block(const float *__restrict__ m, const float *__restrict
     return part;
 }
 
-// threads of a pixel and components kept by each for ns components (0 kept: too many)
+// threads of a pixel and components kept by each for ns components (0 kept: too many).  Eight groups
+// everywhere left threads without a component, and one warp of eight with the pixels' chains; 2000 x 600,
+// FP64 loop of one thread per pixel / 8 groups / this split: 2 components 121 / 167 / 42 us, 4 160 / 177 /
+// 58 us, 8 268 / 193 / 111 us, 16 492 / 260 / 199 us; collapse of 2 components 101 / 102 / 18 us, 4 178 / 107
+// / 28 us.  From 17 components on fewer groups would keep more than 8 components a thread.
 struct RegSplit {
     int groups, cpt;
 };
 __host__ __device__ constexpr RegSplit reg_split(int ns) {
-    return ns <= 16    ? RegSplit{8, 2}
+    return ns <= 2     ? RegSplit{1, 2}
+           : ns <= 4   ? RegSplit{1, 4}
+           : ns <= 8   ? RegSplit{2, 4}
+           : ns <= 16  ? RegSplit{4, 4}
            : ns <= 32  ? RegSplit{8, 4}
            : ns <= 64  ? RegSplit{8, 8}
            : ns <= 128 ? RegSplit{8, 16}
@@ -419,7 +427,10 @@ void reg_dispatch(int ns, F f) {
         if (r.groups == decltype(g)::value && r.cpt == decltype(c)::value) f(g, c);
     };
     using std::integral_constant;
-    call(integral_constant<int, 8>(), integral_constant<int, 2>());
+    call(integral_constant<int, 1>(), integral_constant<int, 2>());
+    call(integral_constant<int, 1>(), integral_constant<int, 4>());
+    call(integral_constant<int, 2>(), integral_constant<int, 4>());
+    call(integral_constant<int, 4>(), integral_constant<int, 4>());
     call(integral_constant<int, 8>(), integral_constant<int, 4>());
     call(integral_constant<int, 8>(), integral_constant<int, 8>());
     call(integral_constant<int, 8>(), integral_constant<int, 16>());

@@ -56,7 +56,7 @@ def _check(efwi, m, b, bp, sink, tol_phi, tol_g=1e-6):
 
 # phi: pairs of FP32 (2^-47) amplified by at most 2 ns, and the oracle's own FP64 sums
 @pytest.mark.parametrize("kind", ["near", "spread", "signed"])
-@pytest.mark.parametrize("ns", [2, 16, 17, 32, 33, 64, 65, 128, 129, 256, 257])
+@pytest.mark.parametrize("ns", [2, 3, 4, 5, 8, 9, 16, 17, 32, 33, 64, 65, 128, 129, 256, 257])
 def test_ends_of_the_splits(efwi, ns, kind):
     rng, b, bp, sink = _weights(ns, 100 + ns)
     z = rng.standard_normal((ns, NZ, NX))
