@@ -310,7 +310,8 @@ float *slot_s(efwi_lbfgs *h, int k) { return h->S + (long long)k * h->n; }
 float *slot_y(efwi_lbfgs *h, int k) { return h->Y + (long long)k * h->n; }
 
 // out = -H g by the two-loop recursion; H = H_0 (I or D) without stored pairs.  out may be h->d, or
-// the caller's vector (g itself included: it is last read before the first element of out is written).
+// the caller's vector, g itself or overlapping it: with pairs, g is last read before the first element
+// of out is written; without, a shifted overlap goes through h->d.
 void lb_direction(efwi_lbfgs *h, const float *g, float *out, cudaStream_t st) {
     double *rho = h->dev + h->o_rho(), *alpha = h->dev + h->o_alpha(), *beta = h->dev + h->o_beta();
     const float *D = h->has_d ? h->D : nullptr;
@@ -319,10 +320,12 @@ void lb_direction(efwi_lbfgs *h, const float *g, float *out, cudaStream_t st) {
     s.in = g;
     s.out = h->d;
     if (np == 0) {
-        s.out = out;
+        const bool shifted = out != g && out < g + h->n && g < out + h->n;
+        s.out = shifted ? h->d : out;
         s.D = D;
         s.neg = 1;
         step_dev(h, s, st);
+        if (shifted) cudaMemcpyAsync(out, h->d, sizeof(float) * h->n, cudaMemcpyDeviceToDevice, st);
         return;
     }
     int k = h->order[np - 1];

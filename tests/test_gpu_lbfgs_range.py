@@ -1,5 +1,5 @@
 """l-BFGS inner products of vectors that are large where the other is small, so that every product is far
-below the product of the two largest elements."""
+below the product of the two largest elements; directions written over the gradient they are made from."""
 import numpy as np
 import pytest
 import torch
@@ -42,4 +42,23 @@ def test_coefficient_of_a_gradient_of_opposite_magnitude(lbfgs, n):
     d = opt.direction(dev(n, (0.0, 1e27, 0.0))).cpu().numpy()
     # a few FP32 roundings of s, y, g and of each update
     assert np.allclose(d[:2], (-1e19, -2e27), rtol=2.0 ** -20, atol=0) and abs(d[2]) <= 2.0 ** -20
+    opt.close()
+
+
+@pytest.mark.parametrize("pairs", [0, 1])
+@pytest.mark.parametrize("shift", [-5, 4, 70_000])
+def test_direction_over_part_of_its_gradient(lbfgs, pairs, shift):
+    n = 3_000_000
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    buf = torch.randn(n + abs(shift), generator=gen, device="cuda")
+    g = buf[max(-shift, 0):][:n]
+    d = buf[max(shift, 0):][:n]
+    opt = lbfgs(n, m=1)
+    for _ in range(pairs):
+        s = torch.randn(n, generator=gen, device="cuda")
+        assert opt.push(s, 2 * s)
+    ref = opt.direction(g.clone())
+    opt.direction(g, d)
+    assert torch.equal(d, ref)
     opt.close()
