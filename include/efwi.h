@@ -282,7 +282,8 @@ typedef struct efwi_zoi_desc {
  *   EFWI_PREFETCH=0|1     L2 prefetch one tile ahead off / on (else timed)
  *   EFWI_AUTOTUNE_LOG=1   print every timed variant on stderr
  *   EFWI_TEST_FAIL_ALLOC=k  make the k-th workspace allocation fail with
- *                         EFWI_ERR_OOM (tests of the clean-up path)
+ *                         EFWI_ERR_OOM (tests of the clean-up path); -k: only
+ *                         with the first row length tried
  *   EFWI_TEST_TUNE_TIMEOUT=1  let a bounded wait run out while variants are
  *                         timed: EFWI_ERR_TIMEOUT, no plan (tests)         */
 int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *desc);

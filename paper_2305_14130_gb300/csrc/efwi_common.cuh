@@ -10,7 +10,8 @@
 //   which tensor copies of 2-byte snapshot elements need at a multiple of 8 (tiles
 //   start at multiples of 32 columns: GX = 4 modulo 8); pitch =
 //   roundup(NX + 8, 32) leaves >= 4 zero columns on the right and starts every
-//   row, and so every halo box, on a 128-byte line; GZ = 2 zero rows above and
+//   row, and so every halo box, on a 128-byte line (where that does not fit in
+//   memory, roundup(NX + 8, 8)); GZ = 2 zero rows above and
 //   below.  Ghost cells are zero and never written, so the radius-2 staggered
 //   stencils need no bounds checks and the discrete derivative operators are exact
 //   transposes up to sign.

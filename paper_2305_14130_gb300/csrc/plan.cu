@@ -28,8 +28,14 @@ static int fail(efwi_plan *p, int code, const std::string &msg) {
 
 namespace {
 
+// Rows of 32 cells start every row, and so every tile's copies, on a 128-byte line; they take up to 24
+// columns more than rows of 8 (1000 cells and 20 of CPML on each side: 0.8 %; 57 cells: a third), which
+// create_plan falls back to where the workspace does not fit.
+constexpr int kRowCells = 32, kRowCellsMin = 8;
+
 // Workspace allocation of a plan.  EFWI_TEST_FAIL_ALLOC=k makes the k-th allocation
-// (1-based) fail without calling cudaMalloc, to test the out-of-memory path.
+// (1-based) fail without calling cudaMalloc, to test the out-of-memory path; -k only
+// that of the first row length tried.
 struct Alloc {
     efwi_plan *p;
     bool ok = true;
@@ -301,7 +307,9 @@ static void free_plan(efwi_plan *p) {
 
 int efwi_autotune(efwi_plan *p);   // k_fused.cu
 
-extern "C" int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *d) {
+// A plan whose rows are a multiple of `row` cells (8 at least: 2-byte snapshot rows are copied in
+// multiples of 16 bytes).
+static int create_plan(efwi_plan **out, const efwi_plan_desc *d, int row) {
     if (!out) return fail(nullptr, EFWI_ERR_ARG, "out is NULL");
     *out = nullptr;
     if (!d) return fail(nullptr, EFWI_ERR_ARG, "desc is NULL");
@@ -402,7 +410,7 @@ extern "C" int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *d) {
         memset(&sh, 0, sizeof sh);
         sh.P = P; sh.x0 = x0; sh.w = w;
         sh.NX = w + 2 * P; sh.NZ = NZ;
-        sh.pitch = (sh.NX + 8 + 31) / 32 * 32;
+        sh.pitch = (sh.NX + 8 + row - 1) / row * row;
         sh.off = off;
         off += (((long long)(NZ + 2 * EFWI_GZ) * sh.pitch + 63) / 64) * 64;
         sh.psx = psx; psx += (long long)NZ * 2 * P;
@@ -453,6 +461,7 @@ extern "C" int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *d) {
     // (the snapshot slots and the checkpoints come last: their number depends on the
     // checkpoint schedule, which EFWI_CKPT_AUTO chooses from the memory left)
     Alloc A{p};
+    if (A.fail_at < 0) A.fail_at = row == kRowCells ? -A.fail_at : 0;
     const long long F = p->fsz_total;
     p->snap_store = d->snap_store;
     p->ck.store = d->ckpt_store;
@@ -613,6 +622,11 @@ extern "C" int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *d) {
     }
     *out = p;
     return EFWI_OK;
+}
+
+extern "C" int efwi_plan_create(efwi_plan **out, const efwi_plan_desc *d) {
+    const int rc = create_plan(out, d, kRowCells);
+    return rc == EFWI_ERR_OOM ? create_plan(out, d, kRowCellsMin) : rc;
 }
 
 extern "C" int efwi_plan_destroy(efwi_plan *p) {
