@@ -192,6 +192,18 @@ def kernel_bytes(exec_, info, nt):
 # in the proportion of the gradient's schedule.  Any other variant, or a kernel changed since its
 # capture, reports traffic null.
 TRAFFIC_PER_CELL = {
+    # lean forward step (tiles at a stride / from the counter), FP32 velocities / FP16 snapshots of every step
+    ("step", 3, 32, 16, 5, 0, 0): {"pass": 54.94, "keep": 59.81},
+    ("step", 3, 32, 16, 4, 0, 0): {"pass": 56.01, "keep": 61.07},
+    ("step", 3, 32, 16, 5, 0, 1): {"keep": 57.64},
+    ("step", 3, 32, 16, 4, 0, 1): {"keep": 58.95},
+    # lean adjoint step, the same
+    ("adj", 2, 32, 16, 5, 2, 0): 98.09,
+    ("adj", 2, 32, 16, 4, 2, 0): 99.77,
+    ("adj", 2, 32, 16, 5, 2, 1): 93.23,
+    ("adj", 2, 32, 16, 4, 2, 1): 95.12,
+    # the variants below were captured with rows of 1048 cells (now 1056) and without the proxy fence after a
+    # tile, neither of which moves other bytes of the fields
     # forward step, TMA cell pairs, tile 32x16
     ("step", 3, 32, 16, 3, 0, 0): {"pass": 54.51, "keep": 59.79},
     # the same with FP16 snapshots (every step stored, per-thread stores)
