@@ -359,8 +359,13 @@ int efwi_plan_set_zoi(efwi_plan *plan, const efwi_zoi_desc *zoi, efwi_stream_t s
  *   phi_reg = 1/2 eta^2 || (I - S^T S_w) W m~ ||^2,
  *   g      += eta^2 W^T (I - S^T S_w)^T (I - S^T S_w) W m~
  * with W of eq. 11 and S_w of eq. 12, per pixel over the ns components.  The
- * residual (I - S^T S_w) W m~ and its norm are FP64; the gradient increment is
- * FP64 at pixels where some component has its sinkhole and FP32 elsewhere.
+ * sums over the components (mean, residual and its norm) carry the rounding
+ * errors of FP32 additions and products along: about 2^-47 of their terms, at
+ * most 2 ns times that for |residual|^2; components with a sinkhole at the
+ * pixel, and values far from 1 in size, are added in FP64, and phi_reg sums
+ * the pixels in FP64.  The gradient increment is FP64 at pixels where some
+ * component has its sinkhole; elsewhere the residual and the trace term are
+ * rounded to FP32 once each.
  *   m, b, bp   device [ns][nz][nx] FP32; sink device [ns][nz][nx] uint8;
  *              b, bp, sink all NULL: the plan's weights (efwi_plan_set_zoi)
  *   phi_reg    device double (overwritten; FP64 reduction)
@@ -403,7 +408,8 @@ int efwi_regularization_grad_noalloc(int ns, int nx, int nz, const float *m, con
 /* Collapse of an extended field to one physical field, out = S_w W x~
  * (eq. 9: the final model from the extended model; the same operator applied
  * to the per-source gradients is the preconditioned gradient of eq. 15).
- * W of eq. 11 and S_w of eq. 12 act per pixel over the ns components, in FP64.
+ * W of eq. 11 and S_w of eq. 12 act per pixel over the ns components; sums as
+ * in efwi_regularization_grad, without differences between components.
  *   x, b, bp   device [ns][nz][nx] FP32; sink device [ns][nz][nx] uint8
  *   out        device [nz][nx] FP32 (overwritten)
  * No plan and no workspace; EFWI_ERR_ARG on sizes < 1 or NULL pointers.     */
@@ -438,8 +444,10 @@ int efwi_pseudo_hessian(efwi_plan *plan, const float *vp, const float *vs, const
  * A handle owns m pairs (s_i, y_i) of n-element FP32 device vectors plus
  * scratch (about (2m + 5) n floats).  Directions come from the two-loop
  * recursion with H_0 = (s^T y / y^T y) I of the newest pair (I without pairs),
- * or a caller's diagonal guess (efwi_lbfgs_set_h0); inner products are FP64
- * reductions in a fixed order.  The line search (bracketing, then zoom with
+ * or a caller's diagonal guess (efwi_lbfgs_set_h0); inner products are
+ * reductions in a fixed order: eight products in FP32 with their rounding
+ * errors (about 2^-47 of sum |x y|; in FP64 where the factors' sizes range
+ * too far for that), these sums in FP64.  The line search (bracketing, then zoom with
  * safeguarded quadratic interpolation) starts at step 1 (1 / ||d|| on the
  * first iteration, d = -H_0 g) and evaluates the objective
  * through the caller's callback:

@@ -10,7 +10,9 @@
 //     on pairs, and F of a tile pair kept in the registers of the thread that updates it.
 // 32 shots of 1000 x 300: 266 -> 247 us (108 B a cell: 5.0 TB/s, 74 % of the measured HBM bandwidth);
 // FP16 snapshots, 8 shots 75 -> 69 us; 2000 x 600, 4 shots 140 -> 114 us; 200 x 100, one shot
-// 10.5 -> 5.8 us.  Two CTAs of two 46 KB stages fill shared memory; the copies in flight bound it.
+// 10.5 -> 5.8 us.  Two CTAs of two 46 KB stages fill shared memory; the copies in flight bound it.  At the
+// 80 registers that two CTAs of 384 threads leave, edge tiles spill (56 bytes a thread at a stride, 76 with
+// the counter): the CPML memory of a pair and of two frame pairs is alive across the wait.
 #include <algorithm>
 
 #include "adjs_tile.cuh"

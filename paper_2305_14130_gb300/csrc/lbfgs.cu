@@ -4,7 +4,8 @@
 //
 // Vectors (the model x, gradients, the m stored pairs s_i = x_{i+1} - x_i,
 // y_i = g_{i+1} - g_i) are FP32 device arrays of n elements; every inner
-// product is an FP64 reduction with a fixed summation order (deterministic).
+// product is a reduction with a fixed summation order (deterministic): eight
+// products in FP32 with their rounding errors, these sums in FP64 (chunk_dot).
 // The search direction is the two-loop recursion (Nocedal & Wright, Alg. 7.4)
 // with H_0 = gamma I, gamma = s^T y / y^T y of the newest pair, or, when the
 // caller sets a positive diagonal D as the initial guess (the paper hands its
