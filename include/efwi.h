@@ -268,7 +268,9 @@ typedef struct efwi_zoi_desc {
  * precomputes CPML profiles, interpolation weights and tile lists, allocates
  * the workspace and, for EXEC_BATCHED with tile 0x0, runs the tile autotuner.
  * Synchronises the device.  Errors: EFWI_ERR_ARG, EFWI_ERR_CFL, EFWI_ERR_OOM,
- * EFWI_ERR_CUDA (*out is then NULL; the message is in efwi_last_error(NULL)).
+ * EFWI_ERR_CUDA, EFWI_ERR_TIMEOUT (a kernel gave up a bounded wait while
+ * variants were timed); *out is then NULL and the message is in
+ * efwi_last_error(NULL).
  * Environment variables read here (all optional; no effect on results, which
  * are bitwise the same for every variant of one adjoint form):
  *   EFWI_TMA_STAGES=n     the autotuner keeps only n-stage TMA forward variants
